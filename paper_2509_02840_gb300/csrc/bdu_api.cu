@@ -91,6 +91,7 @@ struct bdu_ctx {
   RotStream st;
   int *status;
   unsigned long long *counters;
+  int *sync;           // the chase's ticket counter and progress words
   double *scratch64;  // for conversions in read (mixed form)
   // orthogonality control (mixed form)
   void *cublas;           // created on first use
@@ -115,9 +116,7 @@ struct bdu_ctx {
   cudaStream_t sa;       // applications (lowest priority)
   cudaStream_t sc;       // projections' rotation and chases (highest priority)
   cudaEvent_t ev_call, ev_proj, ev_rot, ev_chase, ev_apply[2];
-  // descriptor workspace of batched updates led by this handle, and a second
-  // stream on which their small items' chases run beside the large ones'
-  cudaStream_t batch_aux;
+  // descriptor workspace of batched updates led by this handle
   void *batch_ws;
   size_t batch_ws_bytes;
   // the captured launch sequence of a plain update, replayed while the rank
@@ -299,7 +298,7 @@ cudaError_t enqueue_probe(bdu_ctx *h, int which, double *dst, cudaStream_t s) {
 }
 
 // ---- overlapped mixed form -------------------------------------------------
-// SMs an overlapped apply leaves to the concurrent chase (its cluster).
+// SMs an overlapped apply leaves to the concurrent chase.
 constexpr int kChaseSMs = 16;
 
 // Enqueues on the apply stream the application of record buffer buf to Q and
@@ -741,7 +740,7 @@ bdu_status run_overlapped(bdu_ctx *h, const double *dB, const double *dC) {
   ChaseArgs a{};
   a.m = m; a.n = n; a.band = bp;
   a.rx = 0; a.Ux = nullptr; a.Vx = nullptr;
-  a.st = h->st; a.status = h->status; a.counters = h->counters;
+  a.st = h->st; a.status = h->status; a.counters = h->counters; a.sync = h->sync;
   a.fast = 1;
   a.engine = h->opt.engine;
   a.step_budget = h->opt.step_budget;
@@ -769,7 +768,7 @@ bool alloc_records(bdu_ctx *h, RotStream &r, int T, int cap, int64_t m, bool mix
 // Resources of the rank-r pipeline: a second record buffer, a chase stream of
 // the greatest priority and an apply stream of the least (so that, when a
 // column's application and the next column's chase become ready together, the
-// chase's cluster is placed first), and events.  Made on the first rank-r
+// chase's blocks are placed first), and events.  Made on the first rank-r
 // update; false when they cannot be (the update then runs column by column).
 bool ensure_pipeline(bdu_ctx *h) {
   if (h->pipe_ok) return true;
@@ -879,7 +878,7 @@ bdu_status enqueue_columns_pipelined(bdu_ctx *h, int64_t r) {
     a.rx = after ? 0 : (int)(r - k - 1);
     a.Ux = a.rx > 0 ? h->U + (k + 1) * m : nullptr;
     a.Vx = a.rx > 0 ? h->V + (k + 1) * n : nullptr;
-    a.st = sb; a.status = h->status; a.counters = h->counters;
+    a.st = sb; a.status = h->status; a.counters = h->counters; a.sync = h->sync;
     a.fast = (h->opt.precision == BDU_MIXED) ? 1 : 0;
     a.engine = h->opt.engine;
     a.step_budget = h->opt.step_budget;
@@ -951,7 +950,7 @@ bdu_status enqueue_update(bdu_ctx *h, const double *dB, const double *dC, int64_
     a.rx = after ? 0 : (int)(r - k - 1);
     a.Ux = a.rx > 0 ? h->U + (k + 1) * m : nullptr;
     a.Vx = a.rx > 0 ? h->V + (k + 1) * n : nullptr;
-    a.st = h->st; a.status = h->status; a.counters = h->counters;
+    a.st = h->st; a.status = h->status; a.counters = h->counters; a.sync = h->sync;
     a.fast = (h->opt.precision == BDU_MIXED) ? 1 : 0;
     a.engine = h->opt.engine;
     a.step_budget = h->opt.step_budget;
@@ -1136,7 +1135,6 @@ void bdu_destroy(bdu_handle h) {
   if (h->stream) cudaStreamSynchronize(h->stream);
   if (h->sa) cudaStreamSynchronize(h->sa);
   if (h->sc) cudaStreamSynchronize(h->sc);
-  if (h->batch_aux) cudaStreamSynchronize(h->batch_aux);
   resolve_timers(h);
   drop_graph(h);
   if (h->cublas) cublasDestroy((cublasHandle_t)h->cublas);
@@ -1144,7 +1142,6 @@ void bdu_destroy(bdu_handle h) {
   for (cudaEvent_t ev : {h->ev_call, h->ev_proj, h->ev_rot, h->ev_chase, h->ev_apply[0], h->ev_apply[1]})
     if (ev) cudaEventDestroy(ev);
   if (h->sa) cudaStreamDestroy(h->sa);
-  if (h->batch_aux) cudaStreamDestroy(h->batch_aux);
   if (h->sc) cudaStreamDestroy(h->sc);
   if (h->probe_host) cudaFreeHost(h->probe_host);
   for (void *p : h->blocks) h->al.put(p);
@@ -1229,9 +1226,9 @@ bdu_status bdu_create(bdu_handle *out, int64_t m, int64_t n, const double *Q, co
     rec_ok = rec_ok && alloc_records(h, h->stb[1], T, cap, m, mixed);
     h->stb[1].tc_ws = h->st.tc_ws;  // the applications of the two buffers never overlap
     h->stb[1].tc_ws_bytes = h->st.tc_ws_bytes;
-    // The chase's thread-block cluster needs 16 free SMs of one GPC: its
-    // stream outranks the application's, so that when both become ready the
-    // chase is placed first and the application fills the other SMs.
+    // The chase's stream outranks the application's, so that when both become
+    // ready the chase's blocks are placed first and the application fills the
+    // rest of the GPU.
     int least = 0, greatest = 0;
     cudaDeviceGetStreamPriorityRange(&least, &greatest);
     if (cudaStreamCreateWithPriority(&h->sa, cudaStreamNonBlocking, least) != cudaSuccess ||
@@ -1250,6 +1247,7 @@ bdu_status bdu_create(bdu_handle *out, int64_t m, int64_t n, const double *Q, co
   }
   h->status = (int *)dev_alloc(h, sizeof(int) * 4);
   h->counters = (unsigned long long *)dev_alloc(h, sizeof(unsigned long long) * 16);
+  h->sync = (int *)dev_alloc(h, sizeof(int) * chase_sync_ints((int)m, (int)n));
   h->ortho[0] = h->ortho[1] = -1.0;
   h->ortho_ws = (double *)dev_alloc(h, sizeof(double) * (3 * m + 8));
   if (o.precision == BDU_MIXED) {
@@ -1262,7 +1260,7 @@ bdu_status bdu_create(bdu_handle *out, int64_t m, int64_t n, const double *Q, co
       return BDU_ENOMEM;
     }
   }
-  bool ok = h->Q && h->P && h->band && rec_ok && h->status && h->counters && h->ortho_ws &&
+  bool ok = h->Q && h->P && h->band && rec_ok && h->status && h->counters && h->sync && h->ortho_ws &&
             (o.precision == BDU_FP64 || h->scratch64);
   if (!ok) {
     fail(nullptr, BDU_ENOMEM, "bdu_create: device allocation failed (m=%lld n=%lld)", (long long)m, (long long)n);
@@ -1686,18 +1684,14 @@ static bdu_status update_batch_held(bdu_handle *hs, int count, const double *con
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   const int esz = precision == BDU_FP64 ? 8 : 4;
-  if (!h0->batch_aux && cudaStreamCreateWithFlags(&h0->batch_aux, cudaStreamNonBlocking) != cudaSuccess) {
-    h0->batch_aux = nullptr;
-    return cuda_fail(h0, cudaGetLastError(), "creating the batch stream");
-  }
   for (int64_t k = 0; k < max_r; k++) {
-    // small items (one thread block each) first, then large ones (a cluster each)
-    std::vector<ChaseArgs> chase_s, chase_l;
-    std::vector<const double *> ucol_s, ucol_l, vcol_s, vcol_l;
+    std::vector<ChaseArgs> chase;
+    std::vector<const double *> cols, vcols;  // u columns (then v columns), in chase order
     std::vector<ApplyItem> apply;
     std::vector<std::pair<bdu_ctx *, int>> tc_items;  // (handle, side) applied by the blocked apply
     std::vector<int> first;
-    int max_n = 0, max_n_l = 0, max_band = 0, slabs = 0;
+    int max_blocks = 0, slabs = 0;
+    bool extra = false;  // some item's later projections are rotated inside its chase
     size_t smem = 0;
     for (int i = 0; i < count; i++) {
       if (r[i] <= k) continue;
@@ -1709,23 +1703,16 @@ static bdu_status update_batch_held(bdu_handle *hs, int count, const double *con
       a.rx = after ? 0 : (int)(r[i] - k - 1);
       a.Ux = a.rx > 0 ? h->U + (k + 1) * m : nullptr;
       a.Vx = a.rx > 0 ? h->V + (k + 1) * n : nullptr;
-      a.st = h->st; a.status = h->status; a.counters = h->counters;
+      a.st = h->st; a.status = h->status; a.counters = h->counters; a.sync = h->sync;
       a.fast = precision == BDU_MIXED ? 1 : 0;
       a.step_budget = h->opt.step_budget;
-      if (n >= kClusterBatchMinN && chase_cluster_fits(m, n)) {
-        a.engine = 2;
-        chase_l.push_back(a);
-        ucol_l.push_back(h->U + k * m);
-        vcol_l.push_back(h->V + k * n);
-        if (n > max_n_l) max_n_l = n;
-      } else {
-        a.engine = 1;
-        chase_s.push_back(a);
-        ucol_s.push_back(h->U + k * m);
-        vcol_s.push_back(h->V + k * n);
-        if (n > max_n) max_n = n;
-        if ((int)band_doubles(m, n) > max_band) max_band = (int)band_doubles(m, n);
-      }
+      a.nsync = chase_sync_ints(m, n);
+      a.blocks = chase_blocks(m, n);
+      max_blocks = std::max(max_blocks, a.blocks);
+      extra = extra || a.rx > 0;
+      chase.push_back(a);
+      cols.push_back(h->U + k * m);
+      vcols.push_back(h->V + k * n);
       for (int side = 0; side < 2; side++) {
         const int dim = side == 0 ? m : n;
         if (precision == BDU_MIXED && dim >= kBlockedFrom && h->st.tc_ws) {
@@ -1748,37 +1735,15 @@ static bdu_status update_batch_held(bdu_handle *hs, int count, const double *con
         apply.push_back(it);
       }
     }
-    const int ns = (int)chase_s.size(), nl = (int)chase_l.size(), nact = ns + nl;
-    std::vector<ChaseArgs> chase(chase_s);
-    chase.insert(chase.end(), chase_l.begin(), chase_l.end());
-    std::vector<const double *> cols(ucol_s);  // u columns then v columns, in chase order
-    cols.insert(cols.end(), ucol_l.begin(), ucol_l.end());
-    cols.insert(cols.end(), vcol_s.begin(), vcol_s.end());
-    cols.insert(cols.end(), vcol_l.begin(), vcol_l.end());
+    const int nact = (int)chase.size();
+    cols.insert(cols.end(), vcols.begin(), vcols.end());
     first.push_back(slabs);
     ce = cudaMemcpyAsync(d_chase, chase.data(), sizeof(ChaseArgs) * nact, cudaMemcpyHostToDevice, s);
     if (ce == cudaSuccess) ce = cudaMemcpyAsync(d_cols, cols.data(), sizeof(double *) * cols.size(), cudaMemcpyHostToDevice, s);
     if (ce == cudaSuccess) ce = cudaMemcpyAsync(d_apply, apply.data(), sizeof(ApplyItem) * apply.size(), cudaMemcpyHostToDevice, s);
     if (ce == cudaSuccess) ce = cudaMemcpyAsync(d_first, first.data(), sizeof(int) * first.size(), cudaMemcpyHostToDevice, s);
     if (ce == cudaSuccess) ce = launch_stage_batch(d_chase, d_cols, d_cols + nact, nact, s);
-    // the small items' chases on the second stream, beside the large items'
-    cudaEvent_t fork = nullptr, join = nullptr;
-    if (ce == cudaSuccess && ns > 0 && nl > 0) {
-      ce = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
-      if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&join, cudaEventDisableTiming);
-      if (ce == cudaSuccess) ce = cudaEventRecord(fork, s);
-      if (ce == cudaSuccess) ce = cudaStreamWaitEvent(h0->batch_aux, fork, 0);
-    }
-    const cudaStream_t ss = (ns > 0 && nl > 0) ? h0->batch_aux : s;
-    if (ce == cudaSuccess && ns > 0) ce = launch_chase_batch(d_chase, ns, max_n, max_band, precision == BDU_MIXED, ss);
-    if (ce == cudaSuccess && nl > 0)
-      ce = launch_chase_cluster_batch(d_chase + ns, nl, max_n_l, precision == BDU_MIXED, s);
-    if (ce == cudaSuccess && join) {
-      ce = cudaEventRecord(join, h0->batch_aux);
-      if (ce == cudaSuccess) ce = cudaStreamWaitEvent(s, join, 0);
-    }
-    if (fork) cudaEventDestroy(fork);
-    if (join) cudaEventDestroy(join);
+    if (ce == cudaSuccess) ce = launch_chase_batch(d_chase, nact, max_blocks, precision == BDU_MIXED, extra, s);
     // mixed form: each item's later projections, rotated by this round's rotations
     for (int i = 0; i < count && ce == cudaSuccess; i++) {
       bdu_ctx *h = hs[i];

@@ -92,10 +92,13 @@ struct ChaseArgs {
   int rx;
   RotStream st;
   int *status;        // device error word (ERR_* bits)
-  unsigned long long *counters;  // [0..3] left by phase, [4..7] right by phase, [8] steps
+  unsigned long long *counters;  // [0..3] left by phase, [4..7] right by phase, [8] ops of all chases
   int fast;           // 1: fused multiply-add / Newton rotation arithmetic (mixed form)
-  int engine;         // 0: by size, 1: one CTA, 2: thread-block cluster
-  long long step_budget;  // bound on synchronous steps per column; 0: 64 (n + 16) + 4096
+  int engine;         // 1: one thread block; otherwise as many as the column keeps busy
+  int *sync;          // chase_sync_ints(m, n) ints, zero before the launch
+  int nsync;          // (of a batch's item) that number, for the staging kernel to clear
+  int blocks;         // thread blocks (set by launch_chase; of a batch's item, by the caller)
+  long long step_budget;  // bound on the steps of one warp per column; 0: 64 (n + 16) + 4096
 };
 
 // One matrix (Q or P of one factorization) for the batched apply.
@@ -117,9 +120,8 @@ struct ProjItem {
 
 // Launchers (return the launch error, if any).
 cudaError_t launch_chase(const ChaseArgs &a, cudaStream_t s);
-// The cluster chase engine keeps the band in its CTAs' shared memory; false
-// when (m, n) is too large for that (n above about 48000).
-bool chase_cluster_fits(int m, int n);
+int chase_sync_ints(int m, int n);  // size of ChaseArgs::sync
+int chase_blocks(int m, int n);     // thread blocks a column keeps busy
 
 cudaError_t launch_project(int precision, const void *X, int64_t ld, int nrow, int ncol,
                            const double *B, int64_t ldb, int r, double *U, int64_t ldu,
@@ -151,12 +153,8 @@ cudaError_t launch_apply(int precision, void *X, int64_t ld, int nrow, int ncol,
                          int *status = nullptr, int sm_reserve = 0, bool desc_ready = false,
                          int variant = 0, const int *gate = nullptr);
 
-cudaError_t launch_chase_batch(const ChaseArgs *d_items, int count, int max_n, int max_band_doubles,
-                               int fast, cudaStream_t s);
-// In a batch, items with n at or above this size get a thread-block cluster each.
-constexpr int kClusterBatchMinN = 512;
-cudaError_t launch_chase_cluster_batch(const ChaseArgs *d_items, int count, int max_n, int fast,
-                                       cudaStream_t s);
+cudaError_t launch_chase_batch(const ChaseArgs *d_items, int count, int max_blocks, int fast, bool extra,
+                               cudaStream_t s);
 void apply_geometry(int precision, int ncol, size_t smem_cap, int *R, int *csw);
 cudaError_t launch_apply_reg(float *X, int64_t ld, int nrow, int ncol, const RotStream &st, int side,
                              bool with_spike, int *status, int sm_reserve, bool desc_ready, int layout,

@@ -5,30 +5,17 @@
 // starts with one rotation and pushes the bulge it creates down the band.
 // Chases are generated in a fixed order (the schedule below) and every chase
 // moves monotonically down the band, so chase t may run concurrently with
-// chase t-1 as long as it stays a few positions behind it.  The engine gives
-// each chase to one thread and advances all runnable chases by one rotation
-// per synchronous step; a chase runs only when the nearest earlier unfinished
-// chase is at least D positions ahead (D = 3 between phase-1 chases, 2 from
-// the last phase-2 chase to a phase-3 one, 4 otherwise).  This keeps every
-// band cell's read/write order identical to the sequential algorithm, so the
-// result equals a one-rotation-at-a-time execution.
-//
-// Two engines share the chase logic:
-//   * one CTA (small n): the band sits in that CTA's shared memory when it
-//     fits, else in global memory; steps are separated by __syncthreads;
-//   * a thread-block cluster of 16 CTAs (large n): the band's rows are
-//     partitioned over the CTAs' shared memories and reached through
-//     distributed shared memory; chases are dealt round-robin to the CTAs, and
-//     steps are separated by cluster barriers.  This multiplies the FP64
-//     throughput available to the chases (GB300 issues about two FP64 FMAs
-//     per SM per clock).
+// chase t-1 as long as it stays a few positions behind it: 3 between
+// neighbouring phase-1 chases, 4 otherwise.  This keeps every band cell's
+// read/write order that of the sequential algorithm, so the result equals a
+// one-rotation-at-a-time execution.
 //
 // Schedule (1-based; N = n+1 if m > n else n):
-//   spike:    j = m..n+2: left (j-1, j) zeroing u(j)             [one thread]
+//   spike:    j = m..n+2: left (j-1, j) zeroing u(j)              [one warp]
 //   phase 1:  chase P1(j), j = N..2: left (j-1, j) zeroing u(j); then for
 //             i = j-1, j+1, ...: right (i+1, i+2) zeroing M(i, i+2), left
 //             (i+2, i+3) zeroing M(i+3, i+1), while the bulge exists
-//   fold:     row 1 += u(1) v^T                                   [all threads]
+//   fold:     row 1 += u(1) v^T                                   [one warp]
 //   phase 2:  chase P2(j), j = n..3: right (j-1, j) zeroing M(1, j), then
 //             chase_lower(j-1)
 //   phase 3:  chases P3b(i), P3c(i), i = 1..n-1 (and n when N = n+1):
@@ -38,6 +25,30 @@
 //   chase_lower(k): left (k+1, k+2) zeroing M(k+2, k); right (k+3, k+4)
 //             zeroing M(k+1, k+4); k += 3, while the bulge exists.
 //
+// The engine is a pipeline of groups of kGroup consecutive chases, one thread
+// block a group.  A chase depends on earlier chases only, and only through
+// rows that they have passed, so everything flows one way: a block loads the
+// rows of the band behind the previous group's last chase into a circular
+// window in its shared memory, its chases run there, and the rows behind its
+// own last chase go back to global memory for the next group.  One word per
+// group says up to which row all groups so far are done (release / acquire);
+// its latency is paid once per kGroup chases, not on every step, and no block
+// waits for a slower one behind it.  (Before, all chases of a column advanced
+// together, one rotation per cluster barrier: 3.0 us a step at n = 4096, of
+// which the FP64 sequence was a third.)
+//
+// Inside a block, four warps run the rotations, one per SM sub-partition: on
+// GB300 a warp's FP64 instruction holds its sub-partition's FP64 unit for 64
+// cycles whatever the number of active lanes, so what a step costs is the
+// number of FP64 instructions in one warp's chain.  Each chase therefore has
+// kLanes = 4 lanes: the rotation is computed by all four at once (c, s and r,
+// products or quotients with one factor in common, in one instruction), and
+// each lane rotates one of the up to four pairs: 12 FP64 instructions a step
+// (16 + 10 with a lane per chase).  A fifth warp loads rows, a sixth stores
+// them and publishes the group's word.  Groups are taken from a ticket
+// counter in order, so a block that waits for the group before it waits for
+// one that is already running: any number of resident blocks makes progress.
+//
 // Arithmetic.  Exact (FP64 form): every multiply, add, divide and square root
 // is a separately rounded IEEE operation (__dmul_rn, __dadd_rn, __ddiv_rn,
 // __dsqrt_rn), never a fused multiply-add, so each value is fully determined
@@ -45,33 +56,12 @@
 // multiply-adds, and 1/sqrt(f^2 + g^2) from an FP32 seed refined by one
 // third-order Newton step in FP64 (error well below an FP64 ulp), which
 // avoids the long-latency FP64 division and square-root sequences.
-#include <climits>
-#include <cooperative_groups.h>
-#include <cstdio>
+#include <algorithm>
 
 #include "bdu_internal.cuh"
 
-namespace cg = cooperative_groups;
-
 namespace bdu {
 namespace {
-
-constexpr int kMaxThreads = 256;
-// A placeholder address for band entries outside the stored diagonals: such
-// entries read as zero and their new values are checked (a nonzero one is
-// reported) instead of stored, so it is never read or written.
-__device__ double g_zero_sink[1];
-constexpr int kMaxCluster = 16;
-// Ops a chase may run in one step, each while it stays within the lag of the
-// chase ahead as that chase stood at the start of the step (which only moves
-// further ahead during the step), so any value gives the same results.  Two
-// cut the steps at n = 4096 by a third (45k -> 31k) but made a step 1.66x
-// longer (a warp runs the whole op again for whichever lanes can go on), so
-// the chase took 13% longer: one op per step.
-constexpr int kOpsPerStep = 1;
-
-enum Kind : int { P1 = 0, P2 = 1, P3B = 2, P3C = 3 };
-enum : int { S_L0 = 0, S_R1 = 1, S_L1 = 2, S_A = 3, S_B = 4, S_C = 5, S_CL = 6, S_CR = 7, S_P2 = 8 };
 
 // ----------------------------------------------------------------------------
 // rotation arithmetic
@@ -176,1212 +166,786 @@ template <> struct Arith<true> {
 };
 
 // ----------------------------------------------------------------------------
-// cell stores.  Band cells: dg[j-i+2] at row i >= 2 (offsets -2..3); row 1 is
-// dense (r1[j]); u(1..N), v(1..n).
+// chases, groups, the window
 // ----------------------------------------------------------------------------
-struct LocalStore {
-  double *dg0;  // diagonal o starts at dg0 + (o+2) * ld
-  int ld;
-  double *r1, *u, *v;
-  __device__ __forceinline__ double *cell(int i, int j) const {
-    return (i == 1) ? r1 + j : dg0 + (size_t)(j - i + 2) * ld + i;
-  }
-  static __device__ __forceinline__ double load(const double *p) { return *p; }
-  __device__ __forceinline__ double *uptr(int i) const { return u + i; }
-  __device__ __forceinline__ double *vptr(int j) const { return v + j; }
-  // cell handles of the uniform op: offsets from dg0 (one contiguous buffer)
-  using H = int;
-  __device__ __forceinline__ H h_band(int diag, int i) const { return diag * ld + i; }
-  __device__ __forceinline__ H h_r1(int j) const { return (int)(r1 - dg0) + j; }
-  __device__ __forceinline__ H h_v(int j) const { return (int)(v - dg0) + j; }
-  __device__ __forceinline__ H h_u(int i) const { return (int)(u - dg0) + i; }
-  __device__ __forceinline__ double ld_h(H h) const { return dg0[h]; }
-  __device__ __forceinline__ void st_h(H h, double x) const { dg0[h] = x; }
+constexpr int kLanes = 4;                    // lanes of a chase
+constexpr int kSlots = 32 / kLanes;          // chases of a warp
+constexpr int kRotWarps = 4;                 // warps that rotate (one per SM sub-partition)
+constexpr int kGroup = kRotWarps * kSlots;   // chases of a group
+constexpr int kThreads = 32 * (kRotWarps + 2);
+// Rows of the window.  A group's chases are at most 6 positions apart while
+// none of them has to wait for rows (lag 4, and a position advances by up to
+// 3 at a time), and an op at position p touches rows p-2..p+4.
+constexpr int kWin = 256;
+static_assert(kWin >= 6 * kGroup + 16, "a group's chases must fit the window");
+constexpr int kCells = 9;                    // per row: six diagonals, row 1, v, u
+constexpr int kRowBytes = kCells * 8;        // (an odd number of doubles: no bank conflicts down a column)
+constexpr int kWinBytes = kWin * kRowBytes;
+constexpr int kR1 = 6, kV = 7, kU = 8;       // the last three cells of a row
+constexpr int kPad = 8;                      // rows of zeros below the band
+constexpr int kFar = 1 << 29;                // a position or row beyond every other
+constexpr int kAborted = -1;                 // progress word of a group that gave up
+
+enum : int { S_L0 = 0, S_R1 = 1, S_L1 = 2, S_A = 3, S_B = 4, S_C = 5, S_CL = 6, S_CR = 7, S_P2 = 8 };
+constexpr int kStates = 9;
+
+// Geometry of each op kind.  An op at position a rotates rows (a, a+1) over
+// columns a-dl .. a-dl+w-1, or columns (a, a+1) over as many rows.  src 0: the
+// entry eliminated is the first pair's second, 1: u(a+1) against u(a), 2: row
+// 1's (1, a+1) against (1, a); S_R1 also rotates v(a), v(a+1).  next, dpos:
+// the op that follows while the bulge exists, and its distance; it exists
+// while a + loff <= N (limN) or <= n.
+struct Geo {
+  bool rows;
+  int dl, w, src;
+  bool withv;
+  int next, dpos;
+  bool limN;
+  int loff;
 };
-
-// The band of a thread-block cluster, in distributed shared memory: nine
-// arrays indexed 0..N+1 (the six diagonals by row, row 1 and v by column, u by
-// row), index i of every array held by CTA i % 16 at slot i / 16 of its slice
-// (the same shared-memory offset in every CTA; interleaved, so that the rows
-// the chases are working on are spread over all the CTAs).  An op's cells are
-// reached by their shared::cluster addresses (mapa), the general path's by
-// generic pointers into the cluster's shared-memory window; the cluster
-// barrier between steps orders every CTA's stores before the next step's
-// loads.
-struct DsmStore {
-  double *loc;          // this CTA's slice (generic address)
-  const uint32_t *rb;   // shared::cluster address of every CTA's slice (rb[r] for rank r; in shared memory)
-  int B;                // indices per array and CTA
-  using H = uint32_t;   // a cell's shared::cluster address
-  // (plans also form handles of cells they never touch -- pairs past the
-  // matrix edge, unused slots: harmless, the rank is masked into range and
-  // such a handle is never dereferenced)
-  __device__ __forceinline__ H h_at(int arr, int idx) const {
-    return rb[idx & (kMaxCluster - 1)] + (uint32_t)(arr * B + (idx >> 4)) * 8u;
-  }
-  __device__ __forceinline__ H h_band(int diag, int i) const { return h_at(diag, i); }
-  __device__ __forceinline__ H h_r1(int j) const { return h_at(6, j); }
-  __device__ __forceinline__ H h_v(int j) const { return h_at(7, j); }
-  __device__ __forceinline__ H h_u(int i) const { return h_at(8, i); }
-  __device__ __forceinline__ double ld_h(H h) const {
-    double v;
-    asm volatile("ld.shared::cluster.f64 %0, [%1];\n" : "=d"(v) : "r"(h) : "memory");
-    return v;
-  }
-  __device__ __forceinline__ void st_h(H h, double v) const {
-    asm volatile("st.shared::cluster.f64 [%0], %1;\n" ::"r"(h), "d"(v) : "memory");
-  }
-  __device__ __forceinline__ double *gp(int arr, int idx) const {
-    return static_cast<double *>(__cluster_map_shared_rank(loc + arr * B + (idx >> 4), (unsigned)(idx & (kMaxCluster - 1))));
-  }
-  __device__ __forceinline__ double *cell(int i, int j) const { return (i == 1) ? gp(6, j) : gp(j - i + 2, i); }
-  __device__ __forceinline__ double *uptr(int i) const { return gp(8, i); }
-  __device__ __forceinline__ double *vptr(int j) const { return gp(7, j); }
-  static __device__ __forceinline__ double load(const double *p) { return *p; }
-};
-// Slice of the cluster band per CTA: B indices of each array, 16 B >= N + 2.
-__host__ __device__ inline int dsm_slice(int N) { return (N + 2 + kMaxCluster - 1) / kMaxCluster; }
-
-struct Rec {
-  double *c, *s;
-  int32_t *a;
-  float2 *f;  // FP32 copy of (c, s), or null
-  int cnt, cap;
-  int *err;
-  __device__ __forceinline__ void push(double cc, double ss, int aa) {
-    if (cnt < cap) {
-      a[cnt] = aa;
-      if (c) { c[cnt] = cc; s[cnt] = ss; }
-      if (f) f[cnt] = make_float2(f32_of(cc), f32_of(ss));
-    } else {
-      atomicOr(err, ERR_CAP);
-    }
-    cnt++;
-  }
-};
-
-struct Task {
-  int t;      // task id (>= T: slot exhausted)
-  int kind, p;
-  int st;     // state
-  int ii;     // i (phase 1) or k (chase_lower)
-  int pos;    // position of the next op
-  bool started, done;
-  int phase;  // 1..3, for the rotation counters
-};
-
-__device__ __forceinline__ void task_init(Task &k, int t, int T, int N, int n) {
-  k.t = t;
-  k.started = false;
-  k.done = (t >= T);
-  if (k.done) { k.pos = INT_MAX; return; }
-  int p1 = N - 1, p2 = n > 2 ? n - 2 : 0;
-  if (t < p1) {
-    k.kind = P1; k.p = N - t; k.st = S_L0; k.pos = k.p - 1; k.phase = 1;
-  } else if (t < p1 + p2) {
-    k.kind = P2; k.p = n - (t - p1); k.st = S_P2; k.pos = k.p - 1; k.phase = 2;
-  } else {
-    int q = t - p1 - p2;
-    k.p = q / 2 + 1;
-    k.phase = 3;
-    if ((q & 1) == 0) { k.kind = P3B; k.st = S_A; k.pos = k.p; }
-    else { k.kind = P3C; k.st = S_C; k.pos = k.p + 1; }
-  }
-}
-
-// Geometry of each op kind (the plan in Chaser::run_op), fixed at compile time
-// for the interior of the band.  A row op rotates rows (a, a+1) over columns
-// lo..lo+W-1, a column op columns (a, a+1) over rows lo..lo+W-1; SRC 0: the
-// entry eliminated is the first pair's second, 1: u(a+1) against u(a),
-// 2: row 1's (1, a+1) against (1, a); S_R1 also rotates v(a), v(a+1).  The
-// diagonal (j - i + 2, in 0..5) of the pair's first cell is C + q (rows) or
-// C - q (columns); the second cell's is one less (rows) or one more (columns).
-// Every cell of every kind falls on one of the six stored diagonals.
-struct Geo { bool rows; int w, src; bool withv; int c; };
 __host__ __device__ constexpr Geo geo_of(int st) {
-  return st == S_L0 ? Geo{true, 3, 1, false, 2}
-       : st == S_R1 ? Geo{false, 4, 0, true, 3}
-       : st == S_L1 ? Geo{true, 4, 0, false, 1}
-       : st == S_P2 ? Geo{false, 4, 2, false, 3}
-       : st == S_A  ? Geo{true, 4, 0, false, 2}
-       : st == S_B  ? Geo{false, 5, 0, false, 4}
-       : st == S_C  ? Geo{false, 4, 0, false, 3}
-       : st == S_CL ? Geo{true, 5, 0, false, 1}
-       :              Geo{false, 5, 0, false, 4};  // S_CR
+  return st == S_L0 ? Geo{true, 0, 3, 1, false, S_R1, 1, false, 2}
+       : st == S_R1 ? Geo{false, 1, 4, 0, true, S_L1, 1, true, 2}
+       : st == S_L1 ? Geo{true, 1, 4, 0, false, S_R1, 1, false, 2}
+       : st == S_A  ? Geo{true, 0, 4, 0, false, S_B, 2, false, 3}
+       : st == S_B  ? Geo{false, 2, 5, 0, false, S_CL, 1, true, 2}
+       : st == S_C  ? Geo{false, 1, 4, 0, false, S_CL, 1, true, 2}
+       : st == S_CL ? Geo{true, 1, 5, 0, false, S_CR, 2, false, 3}
+       : st == S_CR ? Geo{false, 2, 5, 0, false, S_CL, 1, true, 2}
+       :              Geo{false, 1, 4, 2, false, S_CL, 1, true, 2};  // S_P2
+}
+// Number of pairs rotated besides the source pair, and which of them holds the
+// bulge (its first cell is the entry the chase looks at next).
+__host__ __device__ constexpr int geo_pairs(int st) {
+  return geo_of(st).w - (geo_of(st).src == 0 ? 1 : 0) + (geo_of(st).withv ? 1 : 0);
+}
+__host__ __device__ constexpr int geo_bulge(int st) { return geo_pairs(st) - 1 - (geo_of(st).withv ? 1 : 0); }
+// info word of a state: bit 0 rows, 1-2 bulge pair, 3-6 next, 7-8 dpos,
+// 9 limN, 10-12 loff, 13 the chase ends when this op finds nothing to rotate
+__host__ __device__ constexpr int geo_info(int st) {
+  return (geo_of(st).rows ? 1 : 0) | geo_bulge(st) << 1 | geo_of(st).next << 3 | geo_of(st).dpos << 7 |
+         (geo_of(st).limN ? 1 : 0) << 9 | geo_of(st).loff << 10 | (st == S_A ? 0 : 1) << 13;
+}
+// Byte offset of cell `cell` of the row `drow` away from the position, from
+// the row two above it (the topmost an op touches).
+__device__ __forceinline__ int rel(int drow, int cell) { return (drow + 2) * kRowBytes + cell * 8; }
+
+// The problem as a sequence of groups: phases 1, 2 and 3 in groups of kGroup
+// chases (no group crosses a phase; phase 1 has one even without chases, since
+// its last group does the fold).
+__host__ __device__ inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
+struct Phases {
+  int N, p1, p2, p3, g1, g2, g3;
+};
+__host__ __device__ inline Phases phases_of(int m, int n) {
+  Phases f;
+  f.N = m > n ? n + 1 : n;
+  f.p1 = f.N - 1;
+  f.p2 = n > 2 ? n - 2 : 0;
+  f.p3 = 2 * (f.N == n + 1 ? n : n - 1);
+  f.g1 = f.p1 > 0 ? ceil_div(f.p1, kGroup) : 1;
+  f.g2 = ceil_div(f.p2, kGroup);
+  f.g3 = ceil_div(f.p3, kGroup);
+  return f;
+}
+// First op (state, position) of chase q (0-based) of a phase.
+__device__ __forceinline__ void first_op(const Phases &F, int n, int phase, int q, int &st, int &pos) {
+  if (phase == 1) { st = S_L0; pos = F.N - q - 1; }
+  else if (phase == 2) { st = S_P2; pos = n - q - 1; }
+  else { st = (q & 1) ? S_C : S_A; pos = q / 2 + 1 + (q & 1); }
 }
 
-// ----------------------------------------------------------------------------
-// the chase logic, shared by both engines
-// ----------------------------------------------------------------------------
-template <class Store, bool FAST>
-struct Chaser {
+// progress words in shared memory (one CTA) and in global memory (the groups)
+__device__ __forceinline__ int ld_cta(const int *p) {
+  int v;
+  asm volatile("ld.acquire.cta.shared.s32 %0, [%1];\n" : "=r"(v) : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_cta(int *p, int v) {
+  asm volatile("st.release.cta.shared.s32 [%0], %1;\n" ::"r"((uint32_t)__cvta_generic_to_shared(p)), "r"(v) : "memory");
+}
+__device__ __forceinline__ int ld_gpu(const int *p) {
+  int v;
+  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_gpu(int *p, int v) {
+  asm volatile("st.release.gpu.global.s32 [%0], %1;\n" ::"l"(p), "r"(v) : "memory");
+}
+
+struct Shared {
+  double win[kWin * kCells];     // cell c of row r at (r mod kWin) * kCells + c
+  int4 tab[kStates * kLanes];    // byte offsets of a lane's cells: source pair, rotated pair (x < 0: none)
+  int info[kStates];
+  int front[kRotWarps];          // position the next warp's first chase stays behind
+  int least[kRotWarps];          // least position of the warp's unfinished chases
+  int loaded;                    // rows up to this one are in the window (kAborted: give up)
+  int flushed;                   // rows up to this one are back in global memory
+  int before;                    // the previous group's word as last read
+  int far;                       // kFar (what the first warp stays behind)
+  int done;                      // rotating warps that have finished the group
+  int loader_done;
+  int ticket;
+};
+
+__device__ __forceinline__ double &cell_at(Shared &S, int off) {
+  return *reinterpret_cast<double *>(reinterpret_cast<char *>(S.win) + off);
+}
+// byte offset of M(i, j) (row 1 dense)
+__device__ __forceinline__ int cell_off(int i, int j) {
+  return i == 1 ? (j & (kWin - 1)) * kRowBytes + kR1 * 8 : (i & (kWin - 1)) * kRowBytes + (j - i + 2) * 8;
+}
+
+__device__ __forceinline__ double make_f64(int hi, unsigned lo) { return __hiloint2double(hi, (int)lo); }
+
+// y ~ 1/sqrt(q), q in [0.25, 2): an FP32 seed (q truncated to FP32 and the
+// seed widened through the bit patterns, about 22 correct bits) refined by
+// y0 (1 + e/2 + 3e^2/8), e = 1 - q y0^2 (third-order Newton step).
+__device__ __forceinline__ double rsqrt_f64(double q) {
+  const unsigned qf = __funnelshift_l((unsigned)__double2loint(q), (unsigned)__double2hiint(q), 3) - (896u << 23);
+  const unsigned u = __float_as_uint(rsqrtf(__uint_as_float(qf)));
+  const double y = make_f64((int)((u >> 3) + (896u << 20)), u << 29);
+  const double e = fma(-(q * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// The rotation of one chase by its four lanes (f, g the same in all of them;
+// every lane of the warp calls it): rotg_fast / rotg_exact, bit for bit.  c
+// and s end up in every lane, r in lanes 2 and 3.
+//
+// Exact: the square root and the two quotients are formed from y ~
+// 1/sqrt(f^2 + g^2) by Newton corrections with exact remainders (Markstein,
+// "IA-64 and Elementary Functions", ch. 8-9), and each is then compared with
+// the rounding interval around it through its exact remainder: h is the
+// rounded root of q iff q - h^2 lies in (-h ulp, h ulp], a quotient the
+// rounded one iff its remainder is below half an ulp of it times h (a tie
+// cannot occur).  18 FP64 instructions against the library's division and
+// square root at n = 1024: 1.7k cycles a step against 5.9k.  The scaling by
+// the larger exponent is exact and does not change any rounding while both
+// inputs lie within 2^-500..2^500 and within 2^900 of each other; for others
+// plain is set, and the caller takes the plain form (rot_plain).
+template <bool FAST>
+__device__ __forceinline__ void rot_lanes(double f, double g, int lane, double &c, double &s, double &r, bool &plain) {
+  const int role = lane & 3;
+  const int fh = __double2hiint(f), gh = __double2hiint(g);
+  const unsigned fl = (unsigned)__double2loint(f), gl = (unsigned)__double2loint(g);
+  const bool fz = ((unsigned)(fh << 1) | fl) == 0, gz = ((unsigned)(gh << 1) | gl) == 0;
+  const int ef = (fh >> 20) & 0x7ff, eg = (gh >> 20) & 0x7ff;
+  const int ex = max(ef, eg), en = min(ef, eg);
+  const int dk = (1022 - ex) << 20;
+  const int sf = fh & (int)0x80000000;
+  if (FAST) {
+    plain = !gz && (ex < 2 || ex > 2044 || (!fz && (en == 0 || en + 1021 < ex)));
+    const double fs = fz ? 0.0 : make_f64(fh + dk, fl), gs = gz ? 0.0 : make_f64(gh + dk, gl);
+    const double q = fma(fs, fs, gs * gs);
+    const double y = rsqrt_f64(q);
+    // c = |fs| y, s = sign(f) gs y and the scaled |r| = q y in one instruction
+    const double a = role == 0 ? fabs(fs) : role == 1 ? make_f64(__double2hiint(gs) ^ sf, (unsigned)__double2loint(gs)) : q;
+    const double pr = a * y;
+    c = __shfl_sync(0xffffffffu, pr, lane & ~3);
+    s = __shfl_sync(0xffffffffu, pr, (lane & ~3) | 1);
+    r = make_f64((__double2hiint(pr) - dk) ^ sf, (unsigned)__double2loint(pr));
+  } else {
+    plain = !gz && !fz && (en < 523 || ex > 1523 || ex - en > 900);
+    const double fs = make_f64((fh & 0x7fffffff) + dk, fl), gs = make_f64((gh & 0x7fffffff) + dk, gl);  // magnitudes
+    const double q = add(mul(fs, fs), mul(gs, gs));
+    const double y = rsqrt_f64(q);
+    const double num = (role & 1) ? gs : fs;
+    const double s0 = q * y, c0 = num * y;
+    const double h1 = fma(fma(-s0, s0, q), make_f64(__double2hiint(y) - (1 << 20), (unsigned)__double2loint(y)), s0);
+    const long long hb = __double_as_longlong(h1);
+    const long long rem = __double_as_longlong(fma(-h1, h1, q));
+    const long long hu = hb + ((long long)((int)(hb >> 52) - (1023 + 52)) << 52);  // h1 times its ulp
+    const long long rmag = rem & 0x7fffffffffffffffLL;
+    int fix = rem >= 0 ? (rmag > hu ? 1 : 0) : (rmag >= hu || hb == 0x3FF0000000000000LL ? -1 : 0);
+    const double h = __longlong_as_double(hb + fix);
+    const double q1 = fma(fma(-c0, h, num), y, c0);
+    const long long qb = __double_as_longlong(q1);
+    const long long qrem = __double_as_longlong(fma(-q1, h, num));
+    long long half = __double_as_longlong(h) + ((long long)((int)(qb >> 52) - (1023 + 53)) << 52);  // h times q1's half ulp
+    if (qrem < 0 && (qb & 0xfffffffffffffLL) == 0) half -= 1LL << 52;  // (below a power of two ulps are half as wide)
+    fix = (qrem & 0x7fffffffffffffffLL) > half ? (qrem < 0 ? -1 : 1) : 0;
+    const double quo = __longlong_as_double(qb + fix);
+    const double oth = __shfl_xor_sync(0xffffffffu, quo, 1);
+    c = (role & 1) ? oth : quo;
+    s = (role & 1) ? quo : oth;
+    s = make_f64(__double2hiint(s) | ((fh ^ gh) & (int)0x80000000), (unsigned)__double2loint(s));
+    r = make_f64((__double2hiint(h) - dk) | sf, (unsigned)__double2loint(h));
+  }
+  c = fz ? 0.0 : c;
+  s = fz ? 1.0 : s;
+  r = fz ? g : r;
+}
+
+template <bool FAST>
+__device__ __noinline__ void rot_plain(double f, double g, double &c, double &s, double &r) {
+  if (FAST) rotg_fast(f, g, c, s, r);
+  else rotg_exact(f, g, c, s, r);
+}
+
+// One op of a chase, as a lane sees it: byte offsets in the window of the
+// source pair (f, g), which becomes (r, 0), and of the lane's own pair; info
+// word of the state, negative when the lane has no pair.
+struct Op {
+  int f, g, x, y, info;
+};
+// (away from row 1)
+__device__ __forceinline__ Op plan_op(Shared &S, int st, int pos, int q) {
+  Op o;
+  const int4 tb = S.tab[st * kLanes + q];
+  o.info = S.info[st] | (tb.w & (int)0x80000000);
+  const int base = ((pos - 2) & (kWin - 1)) * kRowBytes;
+  // offsets past the window's end wrap (as unsigned, the smaller is in range)
+  auto wrap = [](int off) { return (int)min((unsigned)off, (unsigned)(off - kWinBytes)); };
+  o.f = wrap(base + tb.x);
+  o.g = wrap(base + tb.y);
+  o.x = wrap(base + tb.z);
+  o.y = wrap(base + (tb.w & 0xffff));
+  return o;
+}
+// The last position an op touches row 1 from; row 1 is kept apart.
+constexpr int kNearTop = 3;
+__device__ __forceinline__ Op plan_any(Shared &S, int st, int pos, int q) {
+  Op o = plan_op(S, st, pos, q);
+  if (pos <= kNearTop) {
+    if (o.info & 1) {
+      if (pos == 1) {  // S_L0 or S_A: rows 1 and 2, columns from 1 (2) on
+        const int j = pos + q + (st == S_L0 ? 0 : 1);
+        o.x = cell_off(1, j);
+        o.y = cell_off(2, j);
+        if (st == S_A) { o.f = cell_off(1, 1); o.g = cell_off(2, 1); }
+      }
+    } else if (pos - (st == S_B || st == S_CR ? 2 : 1) == 1) {  // columns whose first row is row 1
+      o.f = cell_off(1, pos);
+      o.g = cell_off(1, pos + 1);
+      if (st == S_P2 && q == 0) o.info |= (int)0x80000000;  // (its first band pair is the source pair)
+    }
+  }
+  return o;
+}
+
+// A group's chases, slots kSlots w .. kSlots w + kSlots - 1: warp w.
+//
+// A step's critical path is its FP64 chain; everything else that can be known
+// before the chain ends is computed beside it, for the case that every bulge
+// goes on: the next op and its addresses, whether it may run, what the warp
+// publishes.  When some chase of the warp ends (or skips a step), that is
+// thrown away and recomputed.  (One after the other, at n = 1024: 2.9k cycles
+// a step in the mixed form, of which 1.35k the chain.)
+template <bool FAST, bool EXTRA>
+__device__ __forceinline__ void rotate_chases(const ChaseArgs &Ar, Shared &S, const Phases &F, int phase, int q0, int cnt,
+                                              int w, int max_steps, int &steps, long long max_polls) {
   using A = Arith<FAST>;
-  Store S;
-  int N, n, m;
-  int *err;
-  double *Ux, *Vx;
-  int rx;
-  double *zero;  // placeholder address of entries outside the band (never dereferenced)
-
-  __device__ __forceinline__ bool inband(int i, int j) const {
-    if (i < 1 || i > N || j < 1 || j > n) return false;
-    if (i == 1) return true;
-    const int o = j - i;
-    return o >= -2 && o <= 3;
+  const int lane = threadIdx.x & 31, q = lane & 3, slot = w * kSlots + (lane >> 2);
+  const int n = Ar.n, N = F.N;
+  bool done = slot >= cnt;
+  int st = S_A, pos = kFar;
+  if (!done) first_op(F, n, phase, q0 + slot, st, pos);
+  int eff = done ? 0 : pos;  // what the next chase stays behind
+  // a finished chase passes on what it had to stay behind itself
+  auto relay = [](int ahead) { return ahead >= kFar ? kFar : ahead - 1; };
+  const int lag = phase == 1 ? 3 : 4;
+  const int t = (phase == 1 ? 0 : phase == 2 ? F.p1 : F.p1 + F.p2) + q0 + slot;  // chase number
+  const int cap = Ar.st.cap;
+  // where the lane writes its part of a record: the pair (lane 0), c (1), s (3)
+  char *recL = nullptr, *recR = nullptr;
+  const int stride = q == 0 ? 4 : 8;
+  if (!done) {
+    const size_t rec = (size_t)t * cap;
+    if (q == 0) {
+      recL = reinterpret_cast<char *>(Ar.st.La + rec); recR = reinterpret_cast<char *>(Ar.st.Ra + rec);
+    } else if (FAST) {
+      recL = reinterpret_cast<char *>(Ar.st.Lf + rec) + (q >> 1) * 4;
+      recR = reinterpret_cast<char *>(Ar.st.Rf + rec) + (q >> 1) * 4;
+    } else {
+      recL = reinterpret_cast<char *>((q == 1 ? Ar.st.Lc : Ar.st.Ls) + rec);
+      recR = reinterpret_cast<char *>((q == 1 ? Ar.st.Rc : Ar.st.Rs) + rec);
+    }
   }
-  // an entry outside the band reads as zero without a memory access (a chase's
-  // end test at the bottom of the band would otherwise wait on an L2 round trip)
-  __device__ __forceinline__ double get(int i, int j) const { return inband(i, j) ? Store::load(S.cell(i, j)) : 0.0; }
-  // The later columns of U (V) of a rank-r update: entries (a, a+1) of each
-  // rotated like the band's pair.  Loads of four columns are issued together,
-  // so that they share one L2 round trip.
-  __device__ __forceinline__ void rotate_extra(double *X, int ld, int a, double c, double s) {
-    for (int t0 = 0; t0 < rx; t0 += 4) {
-      double xu[4], yu[4];
-#pragma unroll
-      for (int q = 0; q < 4; q++) {
-        const double *U = X + (size_t)(t0 + q) * ld - 1;
-        xu[q] = t0 + q < rx ? Store::load(U + a) : 0.0;
-        yu[q] = t0 + q < rx ? Store::load(U + a + 1) : 0.0;
+  const int *const before = w > 0 ? &S.front[w - 1] : &S.far;
+  int nl = 0, nr = 0, tried = 0;
+  bool full = false;  // a record did not fit
+  long long polls = 0;
+  int told = -1;  // last published front
+  Op op = plan_any(S, st, done ? 4 : pos, q);
+  bool run = false, any = false;  // may this chase's (some chase's) next op run?
+  for (;;) {
+    __syncwarp();
+    if (!any) {
+      const int pw = ld_cta(before);
+      const int have = ld_cta(&S.loaded);
+      int ahead = __shfl_up_sync(0xffffffffu, eff, kLanes);
+      if (lane < kLanes) ahead = pw;
+      if (done) eff = relay(ahead);
+      run = !done && pos + lag <= ahead && pos + 4 <= have;
+      if (!__any_sync(0xffffffffu, run)) {
+        if (__any_sync(0xffffffffu, have == kAborted)) break;
+        const int last = __shfl_sync(0xffffffffu, eff, 31);
+        if (last != told) {
+          told = last;
+          if (lane == 31) st_cta(&S.front[w], last);
+        }
+        if (last >= kFar && __all_sync(0xffffffffu, done)) break;
+        if (++polls > max_polls) {
+          if (lane == 0) {
+            atomicOr(Ar.status, ERR_STEPS);
+            st_cta(&S.loaded, kAborted);
+          }
+          break;
+        }
+        continue;
       }
-#pragma unroll
-      for (int q = 0; q < 4; q++) {
-        if (t0 + q < rx) {
-          double *U = X + (size_t)(t0 + q) * ld - 1;
-          U[a] = A::px(c, s, xu[q], yu[q]);
-          U[a + 1] = A::py(c, s, xu[q], yu[q]);
+    }
+    const int info = op.info;
+    const bool rows = info & 1, has = info >= 0;
+    const double f = cell_at(S, op.f), g = cell_at(S, op.g);
+    const double x = cell_at(S, op.x), y = cell_at(S, op.y);
+    // later columns of U (V), lane q those of number q, q + kLanes, ...: the
+    // first one's entries are loaded before the rotation
+    double *ex = nullptr;
+    double eu = 0.0, ev = 0.0;
+    if (EXTRA) {
+      const int ldx = rows ? Ar.m : n;
+      if (q < Ar.rx && run && pos < ldx) {
+        ex = (rows ? Ar.Ux : Ar.Vx) + (size_t)q * ldx - 1 + pos;
+        eu = __ldcg(ex);
+        ev = __ldcg(ex + 1);
+      }
+    }
+    const int pw = ld_cta(before);
+    const int have = ld_cta(&S.loaded);
+    // the rotation, and beside it the step after this one for the case that
+    // every bulge goes on (in one basic block, for the compiler to interleave)
+    double c, s, r;
+    bool plain;
+    rot_lanes<FAST>(f, g, lane, c, s, r, plain);
+    const bool exists = pos + ((info >> 10) & 7) <= ((info >> 9) & 1 ? N : n);
+    const int npos = run ? pos + ((info >> 7) & 3) : pos, nst = run ? (info >> 3) & 15 : st;
+    Op nop = plan_op(S, nst, npos, q);
+    int neff = done ? eff : npos;
+    int ahead = __shfl_up_sync(0xffffffffu, neff, kLanes);
+    ahead = lane < kLanes ? pw : ahead;
+    neff = done ? relay(ahead) : neff;
+    const bool nrun = !done && npos + lag <= ahead && npos + 4 <= have;
+    const bool nany = __any_sync(0xffffffffu, nrun);
+    int front = __shfl_sync(0xffffffffu, neff, 31);
+    int least = __reduce_min_sync(0xffffffffu, npos);
+    const bool ok = run && nz(g);
+    const int k = rows ? nl : nr;
+    char *const rp = (rows ? recL : recR) + (size_t)(unsigned)(k * stride);
+    const bool put = ok && k < cap;
+    full = full || (ok && k >= cap);
+    nl += ok && rows ? 1 : 0;
+    nr += ok && !rows ? 1 : 0;
+    tried += run ? 1 : 0;
+    // (scaling extremes; near row 1 the plan above does not hold)
+    const bool top = __any_sync(0xffffffffu, least <= kNearTop);
+    if (__any_sync(0xffffffffu, plain)) {
+      if (plain) rot_plain<FAST>(f, g, c, s, r);
+    }
+    const double nx = A::px(c, s, x, y), ny = A::py(c, s, x, y);
+    if (FAST) {
+      const int v = q == 0 ? pos : __float_as_int(f32_of(q == 1 ? c : s));
+      if (put && q != 2) *reinterpret_cast<int *>(rp) = v;
+    } else {
+      if (put && q == 0) *reinterpret_cast<int *>(rp) = pos;
+      if (put && (q & 1)) *reinterpret_cast<double *>(rp) = q == 1 ? c : s;
+    }
+    if (ok && has) { cell_at(S, op.x) = nx; cell_at(S, op.y) = ny; }
+    if (ok && q == 2) { cell_at(S, op.f) = r; cell_at(S, op.g) = 0.0; }
+    if (EXTRA) {
+      if (ok && ex) {
+        __stcg(ex, A::px(c, s, eu, ev));
+        __stcg(ex + 1, A::py(c, s, eu, ev));
+        for (int kx = q + kLanes; kx < Ar.rx; kx += kLanes) {
+          const int ldx = rows ? Ar.m : n;
+          double *X = (rows ? Ar.Ux : Ar.Vx) + (size_t)kx * ldx - 1 + pos;
+          const double a0 = __ldcg(X), a1 = __ldcg(X + 1);
+          __stcg(X, A::px(c, s, a0, a1));
+          __stcg(X + 1, A::py(c, s, a0, a1));
         }
       }
     }
-  }
-
-  // One rotation, described by its geometry:
-  //   rows (left rotation on rows a, a+1) over columns lo..lo+w-1, or
-  //   cols (right rotation on columns a, a+1) over rows lo..lo+w-1;
-  //   src 0: the entry eliminated is the second of the first pair, i.e.
-  //          (a+1, lo) or (lo, a+1); src 1: u(a+1) against u(a); src 2: row
-  //          1's (1, a+1) against (1, a) (row 1 rotates besides the w rows);
-  //   withv: v(a), v(a+1) rotate too (phase-1 right rotations).
-  // The extra pair (u, row 1 or v) takes the last of the five pair slots,
-  // which these ops leave free (w <= 4 whenever one is needed).  Every lane of
-  // a warp runs the same instruction sequence whatever its op -- on GB300 each
-  // FP64 warp instruction occupies its SM sub-partition's FP64 unit for tens of
-  // cycles however many lanes are active, so lanes must share them: addresses
-  // are formed first (entries outside the band read as zero and their new
-  // values are checked, not stored), all loads are issued together, and the
-  // rotation and the pair updates are branch-free.  Returns false (nothing written) when the entry to
-  // eliminate is already zero; last receives the new value of (a, lo+w-1)
-  // (rows) or (lo+w-1, a) (cols), the bulge the chase looks at next.
-  __device__ __forceinline__ bool exec(bool isrows, int a, int lo, int w, int src, bool withv, Rec &recL,
-                                       Rec &recR, double &last) {
-    // each cell's band test and address are formed once, for its load and its store
-    double *pa[5], *pb[5];
-    bool ia[5], ib[5];  // the cell is stored (inside the band)
-    double x[5], y[5];
-    const bool extra = (src != 0) || withv;
-#pragma unroll
-    for (int q = 0; q < 5; q++) {
-      const bool in = q < w;
-      const int i0 = isrows ? a : lo + q, j0 = isrows ? lo + q : a;
-      const int i1 = isrows ? a + 1 : lo + q, j1 = isrows ? lo + q : a + 1;
-      ia[q] = in && inband(i0, j0);
-      ib[q] = in && inband(i1, j1);
-      pa[q] = ia[q] ? S.cell(i0, j0) : zero;
-      pb[q] = ib[q] ? S.cell(i1, j1) : zero;
-    }
-    if (extra) {
-      if (src == 1) { pa[4] = S.uptr(a); pb[4] = S.uptr(a + 1); }
-      else if (src == 2) { pa[4] = S.cell(1, a); pb[4] = S.cell(1, a + 1); }
-      else { pa[4] = S.vptr(a); pb[4] = S.vptr(a + 1); }
-      ia[4] = ib[4] = true;
-    }
-#pragma unroll
-    for (int q = 0; q < 5; q++) {
-      x[q] = ia[q] ? Store::load(pa[q]) : 0.0;
-      y[q] = ib[q] ? Store::load(pb[q]) : 0.0;
-    }
-    const double f = src == 0 ? x[0] : x[4], g = src == 0 ? y[0] : y[4];
-    double c, s, r;
-    if (!A::rot(f, g, c, s, r)) return false;
-#pragma unroll
-    for (int q = 0; q < 5; q++) {
-      const double nx = A::px(c, s, x[q], y[q]), ny = A::py(c, s, x[q], y[q]);
-      x[q] = nx; y[q] = ny;
-    }
-    if (src == 0) { x[0] = r; y[0] = 0.0; }
-    else { x[4] = r; y[4] = 0.0; }
-    // a value that lands outside the band must be zero (reported otherwise)
-    bool outside = false;
-#pragma unroll
-    for (int q = 0; q < 5; q++) {
-      if (ia[q]) *pa[q] = x[q];
-      else outside |= nz(x[q]);
-      if (ib[q]) *pb[q] = y[q];
-      else outside |= nz(y[q]);
-    }
-    if (outside) atomicOr(err, ERR_BAND);
-    if (isrows) {
-      rotate_extra(Ux, m, a, c, s);
-      recL.push(c, s, a);
+    const unsigned bulges = __ballot_sync(0xffffffffu, ok && has && nz(nx));
+    const bool bulge = (bulges >> ((lane & ~3) + ((info >> 1) & 3))) & 1;
+    const bool on = exists && (bulge || !((info >> 13) & 1));
+    if (__all_sync(0xffffffffu, on || !run) && !top) {
+      pos = npos;
+      st = nst;
+      op = nop;
+      eff = neff;
+      run = nrun;
+      any = nany;
     } else {
-      rotate_extra(Vx, n, a, c, s);
-      recR.push(c, s, a);
-    }
-    last = w == 3 ? x[2] : (w == 4 ? x[3] : x[4]);
-    return true;
-  }
-
-  // exec for an op of kind ST away from row 1 (rows a, a+1 >= 2 for a row
-  // op, lo >= 2 for a column op) whose rotated pair lies inside the matrix:
-  // the same arithmetic on the same values as exec, with the geometry fixed
-  // at compile time.  Cell addresses are a base row plus constant diagonal
-  // offsets; a cell is read and written only inside the matrix (column
-  // lo + q <= n for a row op, row lo + q <= N for a column op), since both
-  // cells of a pair lie on the same side of that bound; pairs whose results
-  // are replaced by (r, 0) are not rotated.
-  template <int ST>
-  __device__ __forceinline__ bool exec_st(int a, int lo, Rec &recL, Rec &recR, double &last) {
-    constexpr Geo G = geo_of(ST);
-    constexpr int W = G.w;
-    constexpr bool EXTRA = G.src != 0 || G.withv;
-    const int lim = (G.rows ? n : N) - lo;  // cell q is inside iff q <= lim
-    double *const base = S.dg0 + (G.rows ? a : lo);
-    const size_t ld = (size_t)S.ld;
-    double *pa[W], *pb[W];
-    double x[W], y[W];
-#pragma unroll
-    for (int q = 0; q < W; q++) {
-      const int oa = G.rows ? G.c + q : G.c - q;
-      const int ob = G.rows ? oa - 1 : oa + 1;
-      pa[q] = base + oa * ld + (G.rows ? 0 : q);
-      pb[q] = base + ob * ld + (G.rows ? 1 : q);
-    }
-    double *pe = nullptr;
-    double xe = 0.0, ye = 0.0;
-    if (EXTRA) pe = G.src == 1 ? S.uptr(a) : (G.src == 2 ? S.cell(1, a) : S.vptr(a));
-#pragma unroll
-    for (int q = 0; q < W; q++) {
-      const bool in = q <= lim;
-      x[q] = in ? Store::load(pa[q]) : 0.0;
-      y[q] = in ? Store::load(pb[q]) : 0.0;
-    }
-    if (EXTRA) { xe = Store::load(pe); ye = Store::load(pe + 1); }
-    const double f = G.src == 0 ? x[0] : xe, g = G.src == 0 ? y[0] : ye;
-    double c, s, r;
-    if (!A::rot(f, g, c, s, r)) return false;
-#pragma unroll
-    for (int q = (G.src == 0 ? 1 : 0); q < W; q++) {
-      const double nx = A::px(c, s, x[q], y[q]), ny = A::py(c, s, x[q], y[q]);
-      x[q] = nx; y[q] = ny;
-    }
-    if (G.src == 0) { x[0] = r; y[0] = 0.0; }
-    if (G.withv) {
-      const double nx = A::px(c, s, xe, ye), ny = A::py(c, s, xe, ye);
-      xe = nx; ye = ny;
-    } else if (G.src != 0) {
-      xe = r; ye = 0.0;
-    }
-#pragma unroll
-    for (int q = 0; q < W; q++) {
-      if (q <= lim) { *pa[q] = x[q]; *pb[q] = y[q]; }
-    }
-    if (EXTRA) { pe[0] = xe; pe[1] = ye; }
-    if (G.rows) {
-      rotate_extra(Ux, m, a, c, s);
-      recL.push(c, s, a);
-    } else {
-      rotate_extra(Vx, n, a, c, s);
-      recR.push(c, s, a);
-    }
-    last = x[W - 1];
-    return true;
-  }
-
-  __device__ __forceinline__ void chase_start(Task &k, int kk, double bulge) {
-    k.ii = kk;
-    if (kk + 2 <= N && nz(bulge)) {
-      k.st = S_CL;
-      k.pos = kk + 1;
-    } else {
-      k.done = true;
-    }
-  }
-
-  // Geometry of the next op of task k (integer logic): the pair (a, a+1) it
-  // rotates, its first row or column lo, width w, source and whether v
-  // rotates too; doit is false when the op does not exist (the state then
-  // only advances).
-  __device__ __forceinline__ void op_geometry(const Task &k, bool &isrows, int &a, int &lo, int &w, int &src,
-                                              bool &withv, bool &doit) const {
-    isrows = false; withv = false; doit = true;
-    a = 0; lo = 0; w = 4; src = 0;
-    switch (k.st) {
-      case S_L0: isrows = true; a = k.p - 1; lo = a; w = 3; src = 1; break;                    // left (j-1, j) on u
-      case S_R1: a = k.ii + 1; lo = k.ii; w = 4; withv = true; break;                            // right (i+1, i+2)
-      case S_L1: isrows = true; a = k.ii + 2; lo = k.ii + 1; w = 4; break;                       // left (i+2, i+3)
-      case S_P2: a = k.p - 1; if (a - 1 == 1) { lo = 1; } else { lo = a - 1; src = 2; } w = 4; break;  // right (j-1, j), row 1
-      case S_A: isrows = true; a = k.p; lo = a; w = 4; doit = (k.p + 1 <= N); break;             // left (i, i+1)
-      case S_B: a = k.p + 2; lo = k.p; w = 5; break;                                             // right (i+2, i+3)
-      case S_C: a = k.p + 1; lo = k.p; w = 4; doit = (k.p + 2 <= n); break;                      // right (i+1, i+2)
-      case S_CL: isrows = true; a = k.ii + 1; lo = k.ii; w = 5; break;                           // left (k+1, k+2)
-      case S_CR: a = k.ii + 3; lo = k.ii + 1; w = 5; break;                                      // right (k+3, k+4)
-    }
-  }
-
-  // Runs one op of task k: the geometry of its next rotation (integer logic),
-  // the rotation itself, then the chase's next state.  Left rotations go to
-  // recL, right ones to recR.
-  __device__ __forceinline__ void run_op(Task &k, Rec &recL, Rec &recR, int &nl, int &nr) {
-    bool isrows, withv, doit;
-    int a, lo, w, src;
-    op_geometry(k, isrows, a, lo, w, src, withv, doit);
-    double b = 0.0;
-    bool ok = false;
-    if (doit) {
-      const bool interior = isrows ? (a >= 2 && a + 1 <= N) : (lo >= 2 && a + 1 <= n);
-      if (!interior) {
-        ok = exec(isrows, a, lo, w, src, withv, recL, recR, b);
-      } else {
-        switch (k.st) {
-          case S_L0: ok = exec_st<S_L0>(a, lo, recL, recR, b); break;
-          case S_R1: ok = exec_st<S_R1>(a, lo, recL, recR, b); break;
-          case S_L1: ok = exec_st<S_L1>(a, lo, recL, recR, b); break;
-          case S_P2: ok = exec_st<S_P2>(a, lo, recL, recR, b); break;
-          case S_A: ok = exec_st<S_A>(a, lo, recL, recR, b); break;
-          case S_B: ok = exec_st<S_B>(a, lo, recL, recR, b); break;
-          case S_C: ok = exec_st<S_C>(a, lo, recL, recR, b); break;
-          case S_CL: ok = exec_st<S_CL>(a, lo, recL, recR, b); break;
-          default: ok = exec_st<S_CR>(a, lo, recL, recR, b); break;
+      __syncwarp();
+      if (run) {
+        if (on) {
+          pos = npos;
+          st = nst;
+        } else if (ok && st == S_R1 && pos + 3 <= n && nz(cell_at(S, cell_off(pos + 1, pos + 3)))) {
+          pos += 2;
+        } else if (ok && st == S_CL && pos + 4 <= N && nz(cell_at(S, cell_off(pos + 4, pos + 2)))) {
+          pos += 3;
+        } else {
+          if (!ok && (st == S_R1 || st == S_L1 || st == S_CL || st == S_CR)) atomicOr(Ar.status, ERR_SCHEDULE);
+          done = true;
+          pos = kFar;
+          if (q == 0) { Ar.st.Ln[t] = nl; Ar.st.Rn[t] = nr; }
         }
       }
+      __syncwarp();
+      eff = done ? eff : pos;
+      ahead = __shfl_up_sync(0xffffffffu, eff, kLanes);
+      ahead = lane < kLanes ? pw : ahead;
+      if (done) eff = relay(ahead);  // (at once, or the chase behind it would lose steps)
+      op = plan_any(S, st, done ? 4 : pos, q);
+      any = false;
+      front = __shfl_sync(0xffffffffu, eff, 31);
+      least = __reduce_min_sync(0xffffffffu, pos);
     }
-    // Keeps the band loads of the advance step (the next bulge) from being
-    // scheduled into the rotation above (measured: ~15% of the step time).
-    asm volatile("" ::: "memory");
-    if (ok) { if (isrows) nl++; else nr++; }
-    advance(k, ok, b);
-  }
-
-  // The chase's next state after an op that rotated (ok) and left the bulge b.
-  __device__ __forceinline__ void advance(Task &k, bool ok, double b) {
-    switch (k.st) {
-      case S_L0: {
-        const int i = k.p - 1;
-        k.ii = i; k.st = S_R1;
-        if (!ok || !(i + 2 <= n && nz(b))) { k.done = true; return; }
-        k.pos = i + 1;
-        return;
+    told = front;
+    __syncwarp();
+    if (lane == 31) {
+      st_cta(&S.front[w], front);
+      st_cta(&S.least[w], least);
+    }
+    if (++steps > max_steps) {
+      if (lane == 0) {
+        atomicOr(Ar.status, ERR_STEPS);
+        st_cta(&S.loaded, kAborted);
       }
-      case S_R1: {
-        int i = k.ii;
-        if (!ok) { atomicOr(err, ERR_SCHEDULE); k.done = true; return; }
-        if (i + 3 <= N && nz(b)) { k.st = S_L1; k.pos = i + 2; return; }
-        i += 2; k.ii = i;
-        if (!(i + 2 <= n && nz(get(i, i + 2)))) { k.done = true; return; }
-        k.pos = i + 1;
-        return;
-      }
-      case S_L1: {
-        if (!ok) { atomicOr(err, ERR_SCHEDULE); k.done = true; return; }
-        const int i = k.ii + 2;
-        k.ii = i; k.st = S_R1;
-        if (!(i + 2 <= n && nz(b))) { k.done = true; return; }
-        k.pos = i + 1;
-        return;
-      }
-      case S_P2: chase_start(k, k.p - 1, ok ? b : 0.0); return;
-      case S_A:
-        k.st = S_B;
-        if (k.p + 3 <= n) { k.pos = k.p + 2; return; }
-        k.done = true;
-        return;
-      case S_B:
-        if (!ok) { k.done = true; return; }
-        chase_start(k, k.p + 2, b);
-        return;
-      case S_C:
-        if (!ok) { k.done = true; return; }
-        chase_start(k, k.p + 1, b);
-        return;
-      case S_CL: {
-        const int kk = k.ii;
-        if (!ok) { atomicOr(err, ERR_SCHEDULE); k.done = true; return; }
-        if (kk + 4 <= n && nz(b)) { k.st = S_CR; k.pos = kk + 3; return; }
-        chase_start(k, kk + 3, get(kk + 5, kk + 3));
-        return;
-      }
-      case S_CR:
-        if (!ok) { atomicOr(err, ERR_SCHEDULE); k.done = true; return; }
-        chase_start(k, k.ii + 3, b);
-        return;
+      break;
     }
   }
+  if (full) atomicOr(Ar.status, ERR_CAP);
+  // rotation counts
+  const int sl = __reduce_add_sync(0xffffffffu, q == 0 ? nl : 0);
+  const int sr = __reduce_add_sync(0xffffffffu, q == 0 ? nr : 0);
+  const int sa = __reduce_add_sync(0xffffffffu, q == 0 ? tried : 0);
+  if (lane == 0) {
+    if (sl) atomicAdd(&Ar.counters[phase], (unsigned long long)sl);
+    if (sr) atomicAdd(&Ar.counters[4 + phase], (unsigned long long)sr);
+    if (sa) atomicAdd(&Ar.counters[8], (unsigned long long)sa);
+    __threadfence_block();
+    atomicAdd(&S.done, 1);
+  }
+}
 
-  // Geometry of an interior op by state, for the plan: bit 0 rows, bits 1-3
-  // w, bits 4-5 src, bit 6 withv, bit 7 a counts from ii (else p), bits 8-10
-  // a's offset + 1, bits 11-12 lo's distance below a, bits 13-14 the op's
-  // existence test (1: p + 1 <= N, 2: p + 2 <= n).  The same values as
-  // op_geometry (which the general path keeps).
-  static __device__ __forceinline__ unsigned geo_word(int st) {
-    switch (st) {  // (the compiler turns the constant table into selects)
-      case S_L0: return 1u | 3u << 1 | 1u << 4 | 0u << 8 | 0u << 11;
-      case S_R1: return 0u | 4u << 1 | 1u << 6 | 1u << 7 | 2u << 8 | 1u << 11;
-      case S_L1: return 1u | 4u << 1 | 1u << 7 | 3u << 8 | 1u << 11;
-      case S_A: return 1u | 4u << 1 | 1u << 8 | 0u << 11 | 1u << 13;
-      case S_B: return 0u | 5u << 1 | 3u << 8 | 2u << 11;
-      case S_C: return 0u | 4u << 1 | 2u << 8 | 1u << 11 | 2u << 13;
-      case S_CL: return 1u | 5u << 1 | 1u << 7 | 2u << 8 | 1u << 11;
-      case S_CR: return 0u | 5u << 1 | 1u << 7 | 4u << 8 | 2u << 11;
-      default: return 0u | 4u << 1 | 2u << 4 | 0u << 8 | 1u << 11;  // S_P2
+// Rows into the window, as far as the previous group has finished them and the
+// window has room.
+__device__ __forceinline__ void load_rows(const ChaseArgs &Ar, Shared &S, const Phases &F, int base, const int *prev,
+                                          bool wait_all) {
+  const int lane = threadIdx.x & 31, n = Ar.n, N = F.N, end = N + kPad;
+  int have = base - 1, before = prev ? 0 : kFar;
+  for (;;) {
+    __syncwarp();
+    if (__shfl_sync(0xffffffffu, ld_cta(&S.done), 0) == kRotWarps) break;
+    if (before < kFar) {
+      before = __shfl_sync(0xffffffffu, ld_gpu(prev), 0);
+      if (before == kAborted) {
+        if (lane == 0) st_cta(&S.loaded, kAborted);
+        break;
+      }
+      // phase 2 starts from row 1 as the fold leaves it: nothing is passed on before
+      if (wait_all && before < kFar) continue;
+      if (lane == 0) st_cta(&S.before, before);
+    }
+    int lim = before >= N ? end : before;
+    lim = min(lim, __shfl_sync(0xffffffffu, ld_cta(&S.flushed), 0) + kWin);
+    if (lim <= have) continue;
+    for (int r0 = have + 1; r0 <= lim; r0 += 32) {
+      const int r = r0 + lane;
+      if (r <= lim) {
+        double v[kCells];
+        const bool row = r <= N;
+#pragma unroll
+        for (int o = 0; o < 6; o++) {
+          const int j = r + o - 2;
+          v[o] = row && j >= 1 && j <= n ? __ldcg(Ar.band.dg[o] + r) : 0.0;
+        }
+        v[kR1] = r <= n ? __ldcg(Ar.band.r1 + r) : 0.0;
+        v[kV] = r <= n ? __ldcg(Ar.band.v + r) : 0.0;
+        v[kU] = row ? __ldcg(Ar.band.u + r) : 0.0;
+        double *d = S.win + (r & (kWin - 1)) * kCells;
+#pragma unroll
+        for (int o = 0; o < kCells; o++) d[o] = v[o];
+      }
+    }
+    have = lim;
+    __syncwarp();
+    if (lane == 0) {
+      const int old = ld_cta(&S.loaded);  // (an abort mark set by another warp stays)
+      __threadfence_block();
+      if (old != kAborted) atomicCAS(&S.loaded, old, have);
+    }
+    __syncwarp();
+  }
+  if (lane == 0) st_cta(&S.loader_done, 1);
+}
+
+__device__ __forceinline__ void store_rows(const ChaseArgs &Ar, Shared &S, const Phases &F, int r0, int r1) {
+  const int lane = threadIdx.x & 31, n = Ar.n, N = F.N;
+  for (int r = r0 + lane; r <= r1; r += 32) {
+    const double *d = S.win + (r & (kWin - 1)) * kCells;
+    if (r <= N) {
+#pragma unroll
+      for (int o = 0; o < 6; o++) __stcg(Ar.band.dg[o] + r, d[o]);
+      __stcg(Ar.band.u + r, d[kU]);
+    }
+    if (r <= n) {
+      __stcg(Ar.band.r1 + r, d[kR1]);
+      __stcg(Ar.band.v + r, d[kV]);
     }
   }
+}
 
-  // ---- one instruction sequence for the interior ops of every kind
-  //
-  // An interior op (the exec_st cases) is the pair (f, g) that defines the
-  // rotation plus three or four pairs rotated with it: the band pairs after
-  // the first when the first is the source, all w band pairs otherwise, then
-  // v(a), v(a+1) when v rotates.  The plan holds their addresses (the
-  // store's cell handles), so that the lanes of a warp whose chases are in
-  // different states run one sequence of FP64 instructions (which on GB300
-  // cost the same for 1 or 32 lanes) instead of one per state.  Same
-  // operations on the same values as exec_st.
-  enum : unsigned char { kNoOp = 0, kUniform = 1, kGeneric = 2 };
-  using H = typename Store::H;
-  struct Plan {
-    H xs, ys;        // the pair (f, g); becomes (r, 0)
-    H xo[4], yo[4];  // the rotated pairs
-    int a, lo, w, src;
-    unsigned char kind, nrot, inmask;  // inmask bit q: rotated pair q lies inside the matrix
-    bool rows, withv;
-  };
-  __device__ __forceinline__ void make_plan(const Task &k, Plan &P) const {
-    P.kind = kNoOp;
-    P.nrot = 0;
-    P.inmask = 0;
-    if (k.done) return;
-    const unsigned gw = geo_word(k.st);
-    const unsigned chk = (gw >> 13) & 3;
-    if ((chk == 1 && k.p + 1 > N) || (chk == 2 && k.p + 2 > n)) return;  // the op does not exist
-    P.rows = gw & 1;
-    P.w = (gw >> 1) & 7;
-    P.src = (gw >> 4) & 3;
-    P.withv = (gw >> 6) & 1;
-    P.a = ((gw >> 7) & 1 ? k.ii : k.p) + (int)((gw >> 8) & 7) - 1;
-    P.lo = P.a - (int)((gw >> 11) & 3);
-    const int a = P.a, lo = P.lo;
-    if (!(P.rows ? (a >= 2 && a + 1 <= N) : (lo >= 2 && a + 1 <= n))) {
-      bool doit;
-      op_geometry(k, P.rows, P.a, P.lo, P.w, P.src, P.withv, doit);  // the general path's exact geometry
-      P.kind = kGeneric;
+// Rows the group's last chase has left, back to global memory; then the
+// group's word.  fold: the last group of phase 1.
+template <bool FAST>
+__device__ __forceinline__ void publish_rows(const ChaseArgs &Ar, Shared &S, const Phases &F, int base, const int *prev,
+                                             int *word, bool fold, long long max_polls) {
+  const int lane = threadIdx.x & 31, n = Ar.n;
+  int flushed = base - 1, told = 0;
+  for (;;) {
+    __syncwarp();
+    // (the order of these loads: what is stored below was final before them)
+    const bool all = ld_cta(&S.done) == kRotWarps && ld_cta(&S.loader_done);
+    int least = kFar;
+#pragma unroll
+    for (int w = 0; w < kRotWarps; w++) least = min(least, ld_cta(&S.least[w]));
+    const int have = ld_cta(&S.loaded);
+    const int before = ld_cta(&S.before);
+    const bool bad = have == kAborted;
+    if (__any_sync(0xffffffffu, bad)) {
+      __syncwarp();
+      if (lane == 0) st_gpu(word, kAborted);
       return;
     }
-    P.kind = kUniform;
-    // band pair q: rows (a, a+1) at column lo+q, diagonals c+q and c+q-1; or
-    // columns (a, a+1) at row lo+q, diagonals c-q and c-q+1 (geo_of(st).c)
-    const int c = P.rows ? lo - a + 2 : a - lo + 2;
-    const int lim = (P.rows ? n : N) - lo;  // band pair q lies inside iff q <= lim
-    const int q0 = P.src == 0 ? 1 : 0;
-    const int nb = P.w - q0;
-    if (P.src == 0) {
-      P.xs = P.rows ? S.h_band(c, a) : S.h_band(c, lo);
-      P.ys = P.rows ? S.h_band(c - 1, a + 1) : S.h_band(c + 1, lo);
-    } else {
-      P.xs = P.src == 1 ? S.h_u(a) : S.h_r1(a);
-      P.ys = P.src == 1 ? S.h_u(a + 1) : S.h_r1(a + 1);
-    }
-    unsigned mask = 0;
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-      const int qq = q0 + q;
-      H xo = P.rows ? S.h_band(c + qq, a) : S.h_band(c - qq, lo + qq);
-      H yo = P.rows ? S.h_band(c + qq - 1, a + 1) : S.h_band(c - qq + 1, lo + qq);
-      bool in = q < nb && qq <= lim;
-      if (P.withv && q == nb) { xo = S.h_v(a); yo = S.h_v(a + 1); in = true; }
-      P.xo[q] = xo; P.yo[q] = yo;
-      mask |= in ? (1u << q) : 0u;
-    }
-    P.inmask = (unsigned char)mask;
-    P.nrot = (unsigned char)(nb + (P.withv ? 1 : 0));
-  }
-  // The loads of a uniform op (zeros for lanes without one), issued together.
-  __device__ __forceinline__ void load_plan(const Plan &P, double &f, double &g, double (&x)[4], double (&y)[4]) const {
-    const bool u = P.kind == kUniform;
-    f = u ? S.ld_h(P.xs) : 0.0;
-    g = u ? S.ld_h(P.ys) : 0.0;
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-      const bool in = u && ((P.inmask >> q) & 1);
-      x[q] = in ? S.ld_h(P.xo[q]) : 0.0;
-      y[q] = in ? S.ld_h(P.yo[q]) : 0.0;
-    }
-  }
-  // Every lane of the warp calls this (the fourth pair is skipped when no
-  // active lane has one); lanes with act store.  Returns act && rotated.
-  __device__ __forceinline__ bool exec_uniform(const Plan &P, bool act, double f, double g, double (&x)[4],
-                                               double (&y)[4], double &c, double &s, double &last) {
-    f = act ? f : 0.0;
-    g = act ? g : 0.0;
-    double r;
-    const bool ok = A::rot(f, g, c, s, r) && act;
-#pragma unroll
-    for (int q = 0; q < 3; q++) {
-      const double nx = A::px(c, s, x[q], y[q]), ny = A::py(c, s, x[q], y[q]);
-      x[q] = nx; y[q] = ny;
-    }
-    if (__any_sync(0xffffffffu, act && P.nrot == 4)) {
-      const double nx = A::px(c, s, x[3], y[3]), ny = A::py(c, s, x[3], y[3]);
-      x[3] = nx; y[3] = ny;
-    }
-    if (ok) {
-      S.st_h(P.xs, r);
-      S.st_h(P.ys, 0.0);
-#pragma unroll
-      for (int q = 0; q < 4; q++) {
-        if ((P.inmask >> q) & 1) { S.st_h(P.xo[q], x[q]); S.st_h(P.yo[q], y[q]); }
+    if (!__all_sync(0xffffffffu, all)) {
+      const int lim = __shfl_sync(0xffffffffu, min(min(least - 3, have), flushed + kWin), 0);
+      const int bf = __shfl_sync(0xffffffffu, before, 0);
+      if (lim > flushed) {
+        store_rows(Ar, S, F, flushed + 1, lim);
+        flushed = lim;
+        __syncwarp();
+        if (lane == 0) st_cta(&S.flushed, flushed);
       }
-      if (rx) rotate_extra(P.rows ? Ux : Vx, P.rows ? m : n, P.a, c, s);
+      const int f = min(flushed, bf);
+      if (f > told) {
+        told = f;
+        __syncwarp();
+        if (lane == 0) st_gpu(word, f);
+      }
+      continue;
     }
-    last = (P.nrot == 4 && !P.withv) ? x[3] : x[2];
-    return ok;
+    break;
   }
-};
-
-// Required lead of chase u over chase t (u < t) in positions.
-__device__ __forceinline__ int lag(int ku, int kt, bool adjacent) {
-  if (!adjacent) return 4;
-  if (ku == P1 && kt == P1) return 3;
-  if (ku == P2 && kt == P3B) return 2;
-  return 4;
+  // the group's chases are finished: the rest of its rows, then everything
+  // below is as the groups before leave it
+  store_rows(Ar, S, F, flushed + 1, ld_cta(&S.loaded));
+  __syncwarp();
+  int before = prev ? 0 : kFar;
+  for (long long polls = 0; before < kFar; polls++) {
+    before = __shfl_sync(0xffffffffu, ld_gpu(prev), 0);
+    if (before == kAborted || polls > max_polls) {
+      if (lane == 0) {
+        if (before != kAborted) atomicOr(Ar.status, ERR_STEPS);
+        st_cta(&S.loaded, kAborted);
+        st_gpu(word, kAborted);
+      }
+      return;
+    }
+    if (before < kFar && before > told) {
+      told = before;
+      if (lane == 0) st_gpu(word, before);
+    }
+  }
+  if (fold) {  // row 1 += u(1) v^T
+    __threadfence();
+    __syncwarp();
+    const double u1 = __ldcg(Ar.band.u + 1);
+    for (int j = 1 + lane; j <= n; j += 32)
+      __stcg(Ar.band.r1 + j, Arith<FAST>::px(1.0, u1, __ldcg(Ar.band.r1 + j), __ldcg(Ar.band.v + j)));
+  }
+  __syncwarp();
+  if (lane == 0) st_gpu(word, kFar);
 }
-__device__ __forceinline__ int kind_of(int t, int p1, int p2) {
-  if (t < p1) return P1;
-  if (t < p1 + p2) return P2;
-  return ((t - p1 - p2) & 1) ? P3C : P3B;
-}
 
-// Logical slot l (chases t with (t / CS) % S == l) lives on thread l: the
-// running chases, a window of consecutive ids, stay packed in few warps.  On
-// GB300 an SM's FP64 unit is shared by all its warps and each FP64 warp
-// instruction holds it for about 16 cycles whatever the number of active
-// lanes, so the cost of a step grows with the number of warps that have a
-// running chase, not with the number of chases.
-__device__ __forceinline__ int thread_slot(int th, int) { return th; }
-
-// status word of a slot: x = task id held, y = pos << 2 | started << 1 | done
-__device__ __forceinline__ int2 enc(const Task &k) {
-  int pos = k.done ? 0 : (k.pos > (INT_MAX >> 3) ? (INT_MAX >> 3) : k.pos);
-  return make_int2(k.t, (pos << 2) | (k.started ? 2 : 0) | (k.done ? 1 : 0));
-}
-
-// The spike (m > n): one sequential chain on u in global memory.
+// The spike (m > n): one sequential chain on u in global memory, by one warp:
+// 32 entries of u are loaded together, the running entry stays in a register;
+// lane k holds u (and, of a rank-r update, the later columns k, k + 32, ... of
+// U go through global memory).
 template <bool FAST>
-__device__ void run_spike(const ChaseArgs &Ar, unsigned long long *cnt0) {
+__device__ __forceinline__ void run_spike(const ChaseArgs &Ar) {
   using A = Arith<FAST>;
-  const int m = Ar.m, n = Ar.n;
+  const int m = Ar.m, n = Ar.n, lane = threadIdx.x & 31;
   int ns = 0;
   double *u = Ar.band.u;
-  for (int j = m; j >= n + 2; j--) {
-    double c, s, r;
-    if (!A::rot(u[j - 1], u[j], c, s, r)) continue;
-    u[j - 1] = r;
-    u[j] = 0.0;
-    for (int t = 0; t < Ar.rx; t++) {
-      double *U = Ar.Ux + (size_t)t * m - 1;
-      const double x = U[j - 1], y = U[j];
-      U[j - 1] = A::px(c, s, x, y);
-      U[j] = A::py(c, s, x, y);
-    }
-    Ar.st.Sc[ns] = c; Ar.st.Ss[ns] = s; Ar.st.Sa[ns] = j - 1;
-    if (Ar.st.Sf) Ar.st.Sf[ns] = make_float2(f32_of(c), f32_of(s));
-    ns++;
+  if (m < n + 2) {
+    if (lane == 0) Ar.st.Sn[0] = 0;
+    return;
   }
-  Ar.st.Sn[0] = ns;
-  *cnt0 = ns;
-}
-
-__device__ __forceinline__ void bind_rec(const ChaseArgs &Ar, const Task &k, Rec &recL, Rec &recR) {
-  const int cap = Ar.st.cap;
-  if (k.t < Ar.st.T) {
-    const size_t o = (size_t)k.t * cap;
-    recL.a = Ar.st.La + o;
-    recR.a = Ar.st.Ra + o;
-    recL.c = Ar.st.Lc ? Ar.st.Lc + o : nullptr; recL.s = Ar.st.Ls ? Ar.st.Ls + o : nullptr;
-    recR.c = Ar.st.Rc ? Ar.st.Rc + o : nullptr; recR.s = Ar.st.Rs ? Ar.st.Rs + o : nullptr;
-    recL.f = Ar.st.Lf ? Ar.st.Lf + o : nullptr;
-    recR.f = Ar.st.Rf ? Ar.st.Rf + o : nullptr;
-    recL.cnt = recR.cnt = 0;
-  }
-}
-
-// ----------------------------------------------------------------------------
-// engine 1: one CTA
-// ----------------------------------------------------------------------------
-template <bool FAST>
-__device__ __forceinline__ void engine_cta(const ChaseArgs &Ar, int use_smem) {
-  extern __shared__ double sh[];
-  __shared__ int2 st[2][kMaxThreads];
-  __shared__ int front[3];
-  __shared__ int p1done, ndone;
-  __shared__ unsigned long long cnt[9];
-
-  const int m = Ar.m, n = Ar.n, N = (m > n) ? n + 1 : n;
-  const int S = blockDim.x, me = threadIdx.x;
-  const int T = Ar.st.T;
-  const int p1 = N - 1, p2 = n > 2 ? n - 2 : 0;
-
-  if (me < 9) cnt[me] = 0;
-  __syncthreads();
-  if (me == 0) run_spike<FAST>(Ar, &cnt[0]);
-  __syncthreads();
-
-  __shared__ double zero_cell;
-  if (me == 0) zero_cell = 0.0;
-  Chaser<LocalStore, FAST> K;
-  K.zero = &zero_cell;
-  K.N = N; K.n = n; K.m = m; K.err = Ar.status;
-  K.Ux = Ar.Ux; K.Vx = Ar.Vx; K.rx = Ar.rx;
-  const int64_t nband = 6 * (int64_t)(N + 2) + 2 * (int64_t)(n + 2) + (N + 2);
-  K.S.ld = N + 2;
-  if (use_smem) {
-    double *p = sh;
-    K.S.dg0 = p; p += 6 * (N + 2);
-    K.S.r1 = p; p += n + 2;
-    K.S.v = p; p += n + 2;
-    K.S.u = p;
-    const double *src = Ar.band.dg[0];
-    for (int64_t q = me; q < nband; q += S) sh[q] = src[q];
-  } else {
-    K.S.dg0 = Ar.band.dg[0];
-    K.S.r1 = Ar.band.r1; K.S.v = Ar.band.v; K.S.u = Ar.band.u;
-  }
-
-  const int myslot = thread_slot(me, S);
-  const int pslot = (myslot + S - 1) % S;  // slot of chase t-1 (t = myslot mod S)
-  Task k;
-  task_init(k, myslot, T, N, n);
-  Rec recL, recR;
-  recL.f = recR.f = nullptr;
-  recL.cap = recR.cap = Ar.st.cap;
-  recL.err = recR.err = Ar.status;
-  int nl = 0, nr = 0;
-  bind_rec(Ar, k, recL, recR);
-  st[0][myslot] = enc(k);
-  if (me == 0) {
-    front[0] = 0; front[1] = INT_MAX; front[2] = INT_MAX;
-    p1done = 0; ndone = 0;
-  }
-  bool fold_done = false;
-  const long long max_steps = Ar.step_budget > 0 ? Ar.step_budget : 64LL * (n + 16) + 4096;
-  long long step = 0;
-  for (;; step++) {
-    // Snapshot the shared counters between two barriers: during the step they
-    // are incremented by threads that finish a chase.
-    __syncthreads();
-    const int p1d = p1done, nd = ndone;
-    __syncthreads();
-    if (!fold_done && p1d == p1) {
-      const double u1 = *K.S.uptr(1);
-      for (int j = me + 1; j <= n; j += S) K.S.r1[j] = Arith<FAST>::px(1.0, u1, K.S.r1[j], K.S.v[j]);
-      __syncthreads();
-      fold_done = true;
-    }
-    if (fold_done && nd == T) break;
-    if (step >= max_steps) {
-      if (me == 0) atomicOr(Ar.status, ERR_STEPS);
-      break;
-    }
-    const int rd = step & 1, wr = rd ^ 1;
-    const int f_rd = step % 3, f_wr = (step + 1) % 3, f_reset = (step + 2) % 3;
-    if (me == 0) front[f_reset] = INT_MAX;
-    const int fr = front[f_rd];
-    if (!k.done) {
-      const int t = k.t;
-      bool ok = !(t >= p1 && !fold_done);
-      int reach = INT_MAX;  // last position this chase may reach in this step
+  double run = __ldcg(u + m);  // u(j), as the rotations so far have left it
+  for (int j0 = m; j0 >= n + 2; j0 -= 32) {
+    const int cnt = min(32, j0 - (n + 1));  // rotations (j-1, j), j = j0 .. j0-cnt+1
+    const double mine = lane < cnt ? __ldcg(u + j0 - 1 - lane) : 0.0;  // u(j0 - 1 - lane)
+    double left = 0.0, kc = 0.0, ks = 0.0;  // u(j0 - lane) afterwards; the rotation of j = j0 - lane
+    bool got = false;
+    for (int k = 0; k < cnt; k++) {
+      const int j = j0 - k;
+      const double f = __shfl_sync(0xffffffffu, mine, k);
+      double c = 1.0, s = 0.0, r = 0.0;
+      bool plain;
+      rot_lanes<FAST>(f, run, lane, c, s, r, plain);
+      if (plain) rot_plain<FAST>(f, run, c, s, r);
+      const bool ok = nz(run);
+      r = __shfl_sync(0xffffffffu, r, 2);
+      if (lane == k) {
+        left = ok ? 0.0 : run;
+        kc = c; ks = s; got = ok;
+      }
       if (ok) {
-        const int lim = (t >= p1) ? p1 : 0;
-        const int stop = fr > lim ? fr : lim;
-        const int kt = kind_of(t, p1, p2);
-        for (int u = t - 1; u >= stop; u--) {
-          int2 w = st[rd][u == t - 1 ? pslot : u % S];
-          if (w.x < u) { ok = false; break; }    // its slot still holds an older chase
-          if (w.x > u || (w.y & 1)) continue;    // finished
-          if (!(w.y & 2)) { ok = false; break; } // not started
-          reach = (w.y >> 2) - lag(kind_of(u, p1, p2), kt, u == t - 1);
-          break;
+        for (int x = lane; x < Ar.rx; x += 32) {
+          double *U = Ar.Ux + (size_t)x * m - 1;
+          const double a = U[j - 1], b = U[j];
+          U[j - 1] = A::px(c, s, a, b);
+          U[j] = A::py(c, s, a, b);
         }
       }
-      // Keeps the op's band loads from being scheduled into the look-back
-      // above (measured: about a quarter of the step time at n = 4096).
-      asm volatile("" ::: "memory");
-      for (int rep = 0; rep < kOpsPerStep && ok && k.pos <= reach; rep++) {
-        K.run_op(k, recL, recR, nl, nr);
-        k.started = true;
-        if (k.done) {
-          Ar.st.Ln[t] = nl;
-          Ar.st.Rn[t] = nr;
-          atomicAdd(&cnt[k.phase], (unsigned long long)nl);
-          atomicAdd(&cnt[4 + k.phase], (unsigned long long)nr);
-          if (t < p1) atomicAdd(&p1done, 1);
-          atomicAdd(&ndone, 1);
-          task_init(k, t + S, T, N, n);
-          nl = nr = 0;
-          bind_rec(Ar, k, recL, recR);
-          break;
-        }
+      run = ok ? r : f;
+    }
+    if (lane < cnt) __stcg(u + j0 - lane, left);
+    const unsigned have = __ballot_sync(0xffffffffu, got);
+    if (got) {
+      const int o = ns + __popc(have & ((1u << lane) - 1));
+      Ar.st.Sc[o] = kc; Ar.st.Ss[o] = ks; Ar.st.Sa[o] = j0 - lane - 1;
+      if (Ar.st.Sf) Ar.st.Sf[o] = make_float2(f32_of(kc), f32_of(ks));
+    }
+    ns += __popc(have);
+  }
+  if (lane == 0) {
+    __stcg(u + n + 1, run);
+    Ar.st.Sn[0] = ns;
+    atomicAdd(&Ar.counters[0], (unsigned long long)ns);
+  }
+  __threadfence();
+}
+
+template <bool FAST, bool EXTRA>
+__device__ __forceinline__ void engine(const ChaseArgs &Ar) {
+  __shared__ Shared S;
+  const int me = threadIdx.x, wid = me >> 5;
+  const int m = Ar.m, n = Ar.n;
+  const Phases F = phases_of(m, n);
+  const int groups = F.g1 + F.g2 + F.g3;
+  int *const ticket = Ar.sync, *const words = Ar.sync + 2;
+  for (int e = me; e < kStates * kLanes; e += kThreads) {
+    const int st = e / kLanes, q = e % kLanes;
+    const Geo G = geo_of(st);
+    const int qq = q + (G.src == 0 ? 1 : 0);
+    int4 t;
+    if (G.src == 1) { t.x = rel(0, kU); t.y = rel(1, kU); }
+    else if (G.src == 2) { t.x = rel(0, kR1); t.y = rel(1, kR1); }
+    else if (G.rows) { t.x = rel(0, 2 - G.dl); t.y = rel(1, 1 - G.dl); }
+    else { t.x = rel(-G.dl, G.dl + 2); t.y = rel(-G.dl, G.dl + 3); }
+    if (G.withv && q == geo_pairs(st) - 1) { t.z = rel(0, kV); t.w = rel(1, kV); }
+    else if (G.rows) { t.z = rel(0, qq - G.dl + 2); t.w = rel(1, qq - G.dl + 1); }
+    else { t.z = rel(qq - G.dl, G.dl - qq + 2); t.w = rel(qq - G.dl, G.dl - qq + 3); }
+    if (q >= geo_pairs(st)) { t.z = t.x; t.w = t.y | (int)0x80000000; }
+    S.tab[e] = t;
+  }
+  if (me < kStates) S.info[me] = geo_info(me);
+  const int max_steps = (int)min(Ar.step_budget > 0 ? Ar.step_budget : 64LL * (n + 16) + 4096, 0x7ffffffeLL);
+  // a poll takes tens of nanoseconds at least, a step half a microsecond; the
+  // spike runs before everything else
+  const long long max_polls = 256LL * max_steps + 64LL * (m - n);
+  int steps = 0;
+  if (me == 0) S.far = kFar;
+  for (;;) {
+    __syncthreads();
+    if (me == 0) {
+      S.ticket = atomicAdd(ticket, 1);
+      S.before = S.done = S.loader_done = 0;
+    }
+    __syncthreads();
+    const int s = S.ticket;
+    if (s >= groups) return;
+    const int phase = s < F.g1 ? 1 : s < F.g1 + F.g2 ? 2 : 3;
+    const int q0 = (s - (phase == 1 ? 0 : phase == 2 ? F.g1 : F.g1 + F.g2)) * kGroup;
+    const int cnt = min(kGroup, (phase == 1 ? F.p1 : phase == 2 ? F.p2 : F.p3) - q0);
+    // the first row of the window: two above the topmost first position
+    int st0, p0 = 1;
+    if (cnt > 0) first_op(F, n, phase, phase == 3 ? q0 : q0 + cnt - 1, st0, p0);
+    const int base = max(1, p0 - 2);
+    int *const word = words + s;
+    const int *const prev = s > 0 ? word - 1 : nullptr;
+    if (me < kRotWarps) {
+      S.front[me] = 0;
+      int least = kFar;
+      for (int k = me * kSlots; k < min(cnt, (me + 1) * kSlots); k++) {
+        int a, p;
+        first_op(F, n, phase, q0 + k, a, p);
+        least = min(least, p);
       }
+      S.least[me] = least;
     }
-    {
-      const int mn = __reduce_min_sync(0xffffffffu, k.done ? INT_MAX : k.t);
-      if ((me & 31) == 0 && mn != INT_MAX) atomicMin(&front[f_wr], mn);
+    if (me == 0) {
+      S.loaded = S.flushed = base - 1;
+      if (s == 0) S.before = kFar;
     }
-    st[wr][myslot] = enc(k);
-  }
-  __syncthreads();
-  if (me == 0) {
-    cnt[8] = step;
-    for (int q = 0; q < 9; q++) atomicAdd(&Ar.counters[q], cnt[q]);
-  }
-  if (use_smem) {
-    double *dst = Ar.band.dg[0];
-    for (int64_t q = me; q < nband; q += S) dst[q] = sh[q];
+    if (s == 0 && wid == 0) run_spike<FAST>(Ar);
+    __syncthreads();
+    if (wid < kRotWarps) rotate_chases<FAST, EXTRA>(Ar, S, F, phase, q0, max(cnt, 0), wid, max_steps, steps, max_polls);
+    else if (wid == kRotWarps) load_rows(Ar, S, F, base, prev, s == F.g1);
+    else publish_rows<FAST>(Ar, S, F, base, prev, word, s == F.g1 - 1, max_polls / 8);
+    __syncthreads();
+    if (S.loaded == kAborted) return;
   }
 }
 
-template <bool FAST>
-__global__ void __launch_bounds__(kMaxThreads) k_chase(ChaseArgs Ar, int use_smem) {
-  engine_cta<FAST>(Ar, use_smem);
-}
-
-// Many independent factorizations, one thread block each (the batched update
-// of resident streams): block b runs the one-CTA engine on items[b]; an item
-// whose band does not fit the launch's dynamic shared memory keeps it in
-// global memory.
-template <bool FAST>
-__global__ void __launch_bounds__(kMaxThreads) k_chase_batch(const ChaseArgs *__restrict__ items,
-                                                             size_t smem_bytes) {
-  const ChaseArgs Ar = items[blockIdx.x];
-  const int N = (Ar.m > Ar.n) ? Ar.n + 1 : Ar.n;
-  const size_t need = sizeof(double) * (6 * (size_t)(N + 2) + 2 * (size_t)(Ar.n + 2) + (N + 2));
-  engine_cta<FAST>(Ar, need <= smem_bytes ? 1 : 0);
-}
-
-// ----------------------------------------------------------------------------
-// engine 2: a thread-block cluster
-// ----------------------------------------------------------------------------
-// The band stays in global memory (L2); chase t runs on CTA t % CS, logical
-// slot (t / CS) % S.  Steps are separated by the cluster barrier, split into
-// its arrive (release) and wait (acquire) halves:
-//
-//   wait      every band write and status word of the previous step is
-//             visible cluster-wide;
-//   loads     the status word of chase t-1 and the counters (shared memory)
-//             are read first, then the planned op's band loads are issued at
-//             once (speculatively: a lane whose chase may not run discards
-//             them), so that the look-back overlaps their latency;
-//   look-back may the chase run (lags behind the nearest earlier unfinished
-//             chase, as in the one-CTA engine);
-//   op        the rotation and its pairs, their stores, the chase's next
-//             state;
-//   publish   status words into this CTA's table and the next CTA's mirror
-//             (chase t-1 always lives on the CTA before chase t's), each
-//             warp's counters (chases done, phase-1 chases done, lowest
-//             unfinished chase) into every CTA's inbox;
-//   arrive    (release: waits for the band stores to be performed);
-//   deferred  the rotation record, a finished chase's bookkeeping and the
-//             next task, the plan (cell offsets) of the next op: nothing any
-//             CTA reads before the next barrier.  (Measured at n = 4096: 146
-//             ms per column against 158 with this work before the arrive.)
-//
-// Status words and inbox slots alternate with the step's parity: a slot
-// written in step s is read in step s+1 and rewritten in step s+2 or later,
-// after every reader of step s+1 has arrived.  So every CTA reads the same
-// totals in a step and leaves the loop in the same step.  Totals are at least
-// one step old, which is conservative.
-__device__ __forceinline__ void cluster_arrive() {
-  __syncwarp();
-  asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait() {
-  __syncwarp();
-  asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-}
-constexpr int kMaxWarps = kMaxThreads / 32;
-// The cluster totals (chases done, phase-1 chases done, lowest unfinished
-// chase) are exchanged every kTotalsEvery steps; between exchanges the last
-// values stand, which only delays the fold and the exit by a few steps and
-// makes the look-back scan a few finished chases more.
-constexpr int kTotalsEvery = 8;
-
-template <bool FAST>
-__device__ __forceinline__ void engine_cluster(const ChaseArgs &Ar) {
-  extern __shared__ double bslice[];     // this CTA's slice of the band (DsmStore)
-  __shared__ int2 st[2][kMaxThreads];    // this CTA's chase status words
-  __shared__ int2 pred[2][kMaxThreads];  // mirror of the previous CTA's status words
-  __shared__ int4 inbox[2][kMaxCluster * kMaxWarps];  // every warp's counters (CTA-major): done, p1 done, min unfinished
-  __shared__ unsigned long long cnt[9];
-
-  cg::cluster_group cl = cg::this_cluster();
-  constexpr int CS = kMaxCluster;  // the launch's cluster size; chase t runs on CTA t % CS
-  const int cta = (int)cl.block_rank();
-  const int m = Ar.m, n = Ar.n, N = (m > n) ? n + 1 : n;
-  const int S = blockDim.x, me = threadIdx.x, lane = me & 31, wid = me >> 5;  // S: a power of two
-  const int NW = S / 32;
-  const int T = Ar.st.T;
-  const int p1 = N - 1, p2 = n > 2 ? n - 2 : 0;
-  const int next = (cta + 1) % CS;
-
-  if (me < 9) cnt[me] = 0;
-  __syncthreads();
-  if (cta == 0 && me == 0) run_spike<FAST>(Ar, &cnt[0]);
-  cl.sync();  // spike done (global u)
-
-  using Ch = Chaser<DsmStore, FAST>;
-  Ch K;
-  K.zero = &g_zero_sink[0];
-  static_assert(kMaxCluster == 16, "the slice layout takes index i to CTA i % 16, slot i / 16");
-  const int B = dsm_slice(N);
-  __shared__ uint32_t rbase[kMaxCluster];
-  if (me < CS) {
-    uint32_t r;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(bslice)), "r"(me));
-    rbase[me] = r;
-  }
-  __syncthreads();
-  K.S.loc = bslice; K.S.rb = rbase;
-  K.S.B = B;
-  K.N = N; K.n = n; K.m = m; K.err = Ar.status;
-  // this CTA's slice of the nine arrays: indices cta * B .. cta * B + B - 1
-  const double *gsrc[9] = {Ar.band.dg[0], Ar.band.dg[1], Ar.band.dg[2], Ar.band.dg[3], Ar.band.dg[4],
-                           Ar.band.dg[5], Ar.band.r1, Ar.band.v, Ar.band.u};
-  const int glen[9] = {N + 2, N + 2, N + 2, N + 2, N + 2, N + 2, n + 2, n + 2, N + 2};
-  for (int arr = 0; arr < 9; arr++)
-    for (int q = me; q < B; q += S) {
-      const int idx = q * CS + cta;
-      bslice[arr * B + q] = idx < glen[arr] ? __ldcg(gsrc[arr] + idx) : 0.0;
-    }
-  K.Ux = Ar.Ux; K.Vx = Ar.Vx; K.rx = Ar.rx;
-
-  int2 *pred_next = cl.map_shared_rank(&pred[0][0], next);
-  const int stride = CS * S;
-  const int myslot = thread_slot(me, S);
-  // this thread's chases are t = cta + CS * j with j = myslot (mod S); chase
-  // t-1 sits on the previous CTA in slot j (or j-1 when cta = 0), which is
-  // where that CTA pushes its status word in this CTA's mirror
-  const int pslot = cta > 0 ? myslot : (myslot + S - 1) % S;
-  Task k;
-  task_init(k, cta + CS * myslot, T, N, n);
-  Rec recL, recR;
-  recL.f = recR.f = nullptr;
-  recL.cap = recR.cap = Ar.st.cap;
-  recL.err = recR.err = Ar.status;
-  int nl = 0, nr = 0;
-  bind_rec(Ar, k, recL, recR);
-  st[0][myslot] = enc(k);
-  pred_next[myslot] = enc(k);  // slot 0 of the next CTA's mirror
-  int ndone = 0, np1 = 0;      // this thread's finished chases (all, phase 1)
-  {
-    const int mn = __reduce_min_sync(0xffffffffu, k.done ? INT_MAX : k.t);
-    if (lane < CS) {
-      int4 *ib = cl.map_shared_rank(&inbox[1][cta * NW + wid], lane);
-      *ib = make_int4(0, 0, mn, 0);
-    }
-  }
-  typename Ch::Plan P;
-  K.make_plan(k, P);
-  bool fold_done = false;
-  int sd = 0, sp1 = 0, fr = 0;  // cluster totals, read every kTotalsEvery steps
-  const long long max_steps = Ar.step_budget > 0 ? Ar.step_budget : 64LL * (n + 16) + 4096;
-  long long step = 0;
-  cluster_arrive();
-  for (;; step++) {
-    cluster_wait();  // every write of the previous step is visible cluster-wide
-    const int rd = step & 1, wr = rd ^ 1;
-    const bool totals = (step & (kTotalsEvery - 1)) == 0;
-    const int2 wpred = pred[rd][pslot];  // chase t-1 (local mirror of the previous CTA)
-    int4 iv[kMaxCluster * kMaxWarps / 32];
-    if (totals) {
-      // cluster totals at the end of the previous step (inbox slot wr)
-#pragma unroll
-      for (int q = 0; q < kMaxCluster * kMaxWarps / 32; q++) {
-        const int e = lane + 32 * q;
-        iv[q] = e < CS * NW ? inbox[wr][e] : make_int4(0, 0, INT_MAX, 0);
-      }
-    }
-    double f, g, x[4], y[4];
-    K.load_plan(P, f, g, x, y);
-    if (totals) {
-      int a0 = 0, a1 = 0, a2 = INT_MAX;
-#pragma unroll
-      for (int q = 0; q < kMaxCluster * kMaxWarps / 32; q++) {
-        a0 += iv[q].x; a1 += iv[q].y; a2 = iv[q].z < a2 ? iv[q].z : a2;
-      }
-      sd = __reduce_add_sync(0xffffffffu, a0);
-      sp1 = __reduce_add_sync(0xffffffffu, a1);
-      fr = __reduce_min_sync(0xffffffffu, a2);
-      if (fr == INT_MAX) fr = T;
-      if (!fold_done && sp1 == p1) {
-        // fold: row 1 += u(1) v^T, each CTA over the columns of its slice
-        const double u1 = DsmStore::load(K.S.uptr(1));
-        for (int q = me; q < B; q += S) {
-          const int j = q * CS + cta;
-          if (j >= 1 && j <= n) bslice[6 * B + q] = Arith<FAST>::px(1.0, u1, bslice[6 * B + q], bslice[7 * B + q]);
-        }
-        cl.sync();
-        fold_done = true;
-        K.load_plan(P, f, g, x, y);  // row 1 has changed
-      }
-      if (fold_done && sd == T) break;
-    }
-    if (step >= max_steps) {
-      if (me == 0) atomicOr(Ar.status, ERR_STEPS);
-      break;
-    }
-    bool run = false;
-    const int t = k.t;
-    if (!k.done) {
-      bool ok = !(t >= p1 && !fold_done);
-      int reach = INT_MAX;  // last position this chase may reach in this step
-      if (ok) {
-        const int lim = (t >= p1) ? p1 : 0;
-        const int stop = fr > lim ? fr : lim;
-        const int kt = kind_of(t, p1, p2);
-        for (int u = t - 1; u >= stop; u--) {
-          int2 w;
-          if (u == t - 1) {
-            w = wpred;
-          } else {
-            const int2 *su = cl.map_shared_rank(&st[0][0], u & (CS - 1));
-            w = su[rd * kMaxThreads + ((u / CS) & (S - 1))];
-          }
-          if (w.x < u) { ok = false; break; }
-          if (w.x > u || (w.y & 1)) continue;
-          if (!(w.y & 2)) { ok = false; break; }
-          reach = (w.y >> 2) - lag(kind_of(u, p1, p2), kt, u == t - 1);
-          break;
-        }
-      }
-      run = ok && k.pos <= reach;
-    }
-    // the op: one FP64 instruction sequence for the warp's interior ops, the
-    // general form (ops touching row 1) apart
-    bool rot = false, pend = false;
-    double c = 0.0, sn = 0.0, b = 0.0;
-    if (__any_sync(0xffffffffu, run && P.kind == Ch::kUniform)) {
-      rot = K.exec_uniform(P, run && P.kind == Ch::kUniform, f, g, x, y, c, sn, b);
-      pend = rot;
-    }
-    if (run && P.kind == Ch::kGeneric) rot = K.exec(P.rows, P.a, P.lo, P.w, P.src, P.withv, recL, recR, b);
-    bool fin = false;
-    if (run) {
-      if (rot) { if (P.rows) nl++; else nr++; }
-      K.advance(k, rot, b);
-      k.started = true;
-      if (k.done) {
-        fin = true;
-        ndone++;
-        if (t < p1) np1++;
-      }
-    }
-    // publish
-    const int2 sw = enc(k);  // a finished chase reads as finished
-    st[wr][myslot] = sw;
-    pred_next[wr * kMaxThreads + myslot] = sw;  // push to the next CTA's mirror
-    if (((step + 1) & (kTotalsEvery - 1)) == 0) {  // read in the next step
-      const int wd = __reduce_add_sync(0xffffffffu, ndone);
-      const int wp = __reduce_add_sync(0xffffffffu, np1);
-      // lowest unfinished chase of the warp (a finished chase's slot moves on
-      // to chase t + stride)
-      const int wm = __reduce_min_sync(0xffffffffu, !k.done ? k.t : (fin && t + stride < T ? t + stride : INT_MAX));
-      if (lane < CS) {
-        int4 *ib = cl.map_shared_rank(&inbox[rd][cta * NW + wid], lane);
-        *ib = make_int4(wd, wp, wm, 0);
-      }
-    }
-    cluster_arrive();
-    // deferred
-    if (pend) (P.rows ? recL : recR).push(c, sn, P.a);
-    if (fin) {
-      Ar.st.Ln[t] = nl;
-      Ar.st.Rn[t] = nr;
-      atomicAdd(&cnt[k.phase], (unsigned long long)nl);
-      atomicAdd(&cnt[4 + k.phase], (unsigned long long)nr);
-      task_init(k, t + stride, T, N, n);  // the slot moves on: chase t reads as finished
-      nl = nr = 0;
-      bind_rec(Ar, k, recL, recR);
-    }
-    K.make_plan(k, P);
-  }
-  if (me == 0) {
-    if (cta == 0) cnt[8] = step;
-  }
-  cl.sync();  // every CTA has left the loop; the slices and phase counters are final
-  {
-    double *gdst[9] = {Ar.band.dg[0], Ar.band.dg[1], Ar.band.dg[2], Ar.band.dg[3], Ar.band.dg[4],
-                       Ar.band.dg[5], Ar.band.r1, Ar.band.v, Ar.band.u};
-    for (int arr = 0; arr < 9; arr++)
-      for (int q = me; q < B; q += S) {
-        const int idx = q * CS + cta;
-        if (idx < glen[arr]) gdst[arr][idx] = bslice[arr * B + q];
-      }
-  }
-  if (me == 0) {
-    for (int q = 0; q < 9; q++)
-      if (cnt[q]) atomicAdd(&Ar.counters[q], cnt[q]);
-  }
-}
-
-template <bool FAST>
-__global__ void __launch_bounds__(kMaxThreads) k_chase_cluster(ChaseArgs Ar) {
-  engine_cluster<FAST>(Ar);
-}
-
-// Many independent factorizations, one 16-CTA cluster each (the large items
-// of a batched update): cluster c runs the cluster engine on items[c].
-template <bool FAST>
-__global__ void __launch_bounds__(kMaxThreads) k_chase_cluster_batch(const ChaseArgs *__restrict__ items) {
-  const ChaseArgs Ar = items[blockIdx.x / kMaxCluster];
-  engine_cluster<FAST>(Ar);
-}
-
-// Static shared memory of the cluster engine (status words, mirrors, inbox)
-// with some margin, and its dynamic shared memory: the band slice of each CTA.
-constexpr size_t kClusterStaticSmem = 16384;
-size_t cluster_slice_bytes(int n, int m) {
-  const int N = (m > n) ? n + 1 : n;
-  return (size_t)9 * sizeof(double) * dsm_slice(N);
-}
-
-// Threads per CTA of the cluster engine: a slot for each of the ~n/3 chases in
-// flight, a power of two (64..kMaxThreads) so that slot arithmetic is shifts.
-int cluster_threads(int n) {
-  const int need = (n / 3 + 16) / kMaxCluster;
-  int t = 64;
-  while (t < need && t < kMaxThreads) t *= 2;
-  return t;
-}
-
-template <bool FAST>
-cudaError_t launch_engine(const ChaseArgs &a, cudaStream_t s) {
-  const int n = a.n, m = a.m;
-  const int N = (m > n) ? n + 1 : n;
-  int dev = 0, optin = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  // by size: one CTA up to the measured crossover (n = 512: 17.2 vs 20.0 ms
-  // per mixed column, 26.2 vs 28.0 FP64; n = 1024: 42.9 vs 40.9, 69.4 vs 56.9)
-  const int cluster_from = FAST ? 896 : 640;
-  // the cluster engine holds the band in its CTAs' shared memory (about
-  // 9 (n + 2) / 16 doubles each: n < 48000)
-  const bool fits = cluster_slice_bytes(n, m) + kClusterStaticSmem <= (size_t)optin;
-  if (fits && a.engine != 1 && (a.engine == 2 || n >= cluster_from)) {
-    // cluster engine
-    const int CS = kMaxCluster;
-    const int threads = cluster_threads(n);
-    cudaError_t e = cudaFuncSetAttribute(k_chase_cluster<FAST>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    const size_t dyn = cluster_slice_bytes(n, m);
-    e = cudaFuncSetAttribute(k_chase_cluster<FAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(CS);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = dyn;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CS;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, k_chase_cluster<FAST>, a);
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
-  }
-  int threads = ((n / 3 + 16 + 31) / 32) * 32;
-  if (threads < 32) threads = 32;
-  if (threads > kMaxThreads) threads = kMaxThreads;
-  const size_t smem = sizeof(double) * (6 * (size_t)(N + 2) + 2 * (size_t)(n + 2) + (N + 2));
-  const size_t static_smem = sizeof(int2) * 2 * kMaxThreads + 64 + 9 * 8;
-  const int use_smem = (smem + static_smem + 1024 <= (size_t)optin) ? 1 : 0;
-  const size_t dyn = use_smem ? smem : 0;
-  if (use_smem) {
-    cudaError_t e = cudaFuncSetAttribute(k_chase<FAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-    if (e != cudaSuccess) return e;
-  }
-  k_chase<FAST><<<1, threads, dyn, s>>>(a, use_smem);
-  return cudaGetLastError();
+template <bool FAST, bool EXTRA>
+__global__ void __launch_bounds__(kThreads) k_chase(ChaseArgs Ar) {
+  engine<FAST, EXTRA>(Ar);
 }
 
 }  // namespace
 
-// The items one thread-block cluster each; the block size suits the largest n.
-cudaError_t launch_chase_cluster_batch(const ChaseArgs *d_items, int count, int max_n, int fast,
-                                       cudaStream_t s) {
-  if (count <= 0) return cudaSuccess;
-  const int CS = kMaxCluster;
-  const int threads = cluster_threads(max_n);
-  const size_t dyn = cluster_slice_bytes(max_n, max_n + 1);  // N <= max_n + 1
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(CS * count);
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = dyn;
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = CS;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  cudaError_t e;
-  if (fast) {
-    e = cudaFuncSetAttribute(k_chase_cluster_batch<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_chase_cluster_batch<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, k_chase_cluster_batch<true>, d_items);
-  } else {
-    e = cudaFuncSetAttribute(k_chase_cluster_batch<false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_chase_cluster_batch<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, k_chase_cluster_batch<false>, d_items);
-  }
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+int chase_sync_ints(int m, int n) {
+  const Phases F = phases_of(m, n);
+  return 2 + F.g1 + F.g2 + F.g3;
 }
 
-cudaError_t launch_chase_batch(const ChaseArgs *d_items, int count, int max_n, int max_band_doubles,
-                               int fast, cudaStream_t s) {
-  if (count <= 0) return cudaSuccess;
-  int dev = 0, optin = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  int threads = ((max_n / 3 + 16 + 31) / 32) * 32;
-  if (threads < 32) threads = 32;
-  if (threads > kMaxThreads) threads = kMaxThreads;
-  const size_t static_smem = sizeof(int2) * 2 * kMaxThreads + 256;
-  size_t dyn = sizeof(double) * (size_t)max_band_doubles;
-  if (dyn + static_smem > (size_t)optin) dyn = (size_t)optin - static_smem;
-  cudaError_t e;
-  if (fast) {
-    e = cudaFuncSetAttribute(k_chase_batch<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-    if (e != cudaSuccess) return e;
-    k_chase_batch<true><<<count, threads, dyn, s>>>(d_items, dyn);
-  } else {
-    e = cudaFuncSetAttribute(k_chase_batch<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-    if (e != cudaSuccess) return e;
-    k_chase_batch<false><<<count, threads, dyn, s>>>(d_items, dyn);
-  }
-  return cudaGetLastError();
+// Blocks for a column: enough for the groups in flight.  A phase-1 chase
+// starts about every two steps and runs for up to n of them, so n / (2 kGroup)
+// groups overlap there; two more cover the hand-over between groups.
+int chase_blocks(int m, int n) {
+  const Phases F = phases_of(m, n);
+  return std::min(F.g1 + F.g2 + F.g3, n / (2 * kGroup) + 3);
 }
 
-bool chase_cluster_fits(int m, int n) {
-  int dev = 0, optin = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  return cluster_slice_bytes(n, m) + kClusterStaticSmem <= (size_t)optin;
+namespace {
+
+// Many independent factorizations: blocks (i, .) run items[i] (so that every
+// item has a block in the first wave).
+template <bool FAST, bool EXTRA>
+__global__ void __launch_bounds__(kThreads) k_chase_batch(const ChaseArgs *__restrict__ items) {
+  __shared__ ChaseArgs Ar;  // (in shared memory: a copy in registers halves the blocks an SM holds)
+  if (threadIdx.x == 0) Ar = items[blockIdx.x];
+  __syncthreads();
+  if ((int)blockIdx.y >= Ar.blocks) return;
+  engine<FAST, EXTRA>(Ar);
+}
+
+}  // namespace
+
+cudaError_t launch_chase_batch(const ChaseArgs *d_items, int count, int max_blocks, int fast, bool extra,
+                               cudaStream_t s) {
+  if (count <= 0) return cudaSuccess;
+  const dim3 grid(count, max_blocks);
+  auto *const k = fast ? (extra ? k_chase_batch<true, true> : k_chase_batch<true, false>)
+                       : (extra ? k_chase_batch<false, true> : k_chase_batch<false, false>);
+  k<<<grid, kThreads, 0, s>>>(d_items);
+  return cudaGetLastError();
 }
 
 // Failure injection (BDU_INJECT_STEP_BUDGET) sets the step budget of a
@@ -1390,8 +954,13 @@ cudaError_t launch_chase(const ChaseArgs &a0, cudaStream_t s) {
   ChaseArgs a = a0;
   const Injection inj = injection();
   if (a.step_budget == 0 && inj.site == BDU_INJECT_STEP_BUDGET) a.step_budget = inj.value;
-  return a.fast ? launch_engine<true>(a, s) : launch_engine<false>(a, s);
+  a.blocks = a.engine == 1 ? 1 : chase_blocks(a.m, a.n);
+  const cudaError_t e = cudaMemsetAsync(a.sync, 0, sizeof(int) * chase_sync_ints(a.m, a.n), s);
+  if (e != cudaSuccess) return e;
+  auto *const k = a.fast ? (a.rx > 0 ? k_chase<true, true> : k_chase<true, false>)
+                         : (a.rx > 0 ? k_chase<false, true> : k_chase<false, false>);
+  k<<<a.blocks, kThreads, 0, s>>>(a);
+  return cudaGetLastError();
 }
 
 }  // namespace bdu
-

@@ -37,7 +37,7 @@ constexpr int64_t align256(int64_t x) { return (x + 255) / 256 * 256; }
 
 // Byte layout of the scratch for an m x n problem.
 struct Layout {
-  int64_t band, nz_b, nz_c, Lc, Ls, Rc, Rs, La, Ra, Ln, Rn, Sc, Ss, Sa, Sn, status, counters, total;
+  int64_t band, nz_b, nz_c, Lc, Ls, Rc, Rs, La, Ra, Ln, Rn, Sc, Ss, Sa, Sn, status, counters, sync, total;
 };
 
 constexpr Layout layout(int64_t m, int64_t n) {
@@ -67,6 +67,7 @@ constexpr Layout layout(int64_t m, int64_t n) {
   L.Sn = o; o = align256(o + 16);
   L.status = o; o = align256(o + 16);
   L.counters = o; o = align256(o + 8 * 16);
+  L.sync = o; o = align256(o + 4 * (T / 16 + 8));  // chase_sync_ints: 2 + T / 32 and up to three part groups
   L.total = o;
   return L;
 }
@@ -194,6 +195,7 @@ extern "C" bdu_status bdu_update_rank1_noalloc(int64_t m, int64_t n, double *Q, 
     a.m = (int)m; a.n = (int)n; a.band = bp;
     a.Ux = nullptr; a.Vx = nullptr; a.rx = 0;
     a.st = st; a.status = status; a.counters = counters;
+    a.sync = (int *)(base + L.sync);
     ce = launch_chase(a, s);
   }
   // a failure of the chase (status word nonzero) leaves Q, P, d and e untouched

@@ -138,6 +138,7 @@ __global__ void k_stage_batch(const ChaseArgs *__restrict__ items, const double 
   for (int i = threadIdx.x; i < a.m; i += blockDim.x) a.band.u[i + 1] = uc[i];
   for (int j = threadIdx.x; j < a.n; j += blockDim.x) a.band.v[j + 1] = vc[j];
   for (int t = threadIdx.x; t < a.st.T; t += blockDim.x) { a.st.Ln[t] = 0; a.st.Rn[t] = 0; }
+  for (int t = threadIdx.x; t < a.nsync; t += blockDim.x) a.sync[t] = 0;
 }
 
 }  // namespace

@@ -61,6 +61,7 @@ def reserve_bytes(m, n, precision, max_rank=4):
     else:
         b += tc * (4 * 8 + 2 * 4)                         # FP64 (c, s) and int32 pair records
     b += 8 * (T + 1) + 20 * (m + 1) + 8 * (3 * m + 8) + 256
+    b += 4 * (T // 32 + 8)                                # the chase's progress words
     b += max_rank * (16 * (m + n) + 4 * (m + n)) + 8      # B, C, U, V and their nonzero lists
     if precision == bdu.MIXED:
         b += 8 * m * m + 8 * (m + 1) + 32 * (T + 1)       # FP64 scratch, spike copies, chase descriptors
