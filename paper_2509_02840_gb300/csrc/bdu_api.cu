@@ -593,7 +593,7 @@ bdu_status tune_side(bdu_ctx *h, int side, int sm_reserve) {
   // layouts and the FP32 slab), so that the choice changes no result
   std::vector<int> cand;
   if (!mixed) {
-    for (int R : {2, 4, 6, 8, 10, 12, 16, 20, 24, 32, 48, 64}) cand.push_back(R);
+    for (int R : {2, 3, 4, 5, 6, 7, 8, 9, 11, 13, 16, 20, 24, 32, 48, 64}) cand.push_back(R);
   } else {
     for (int v = 1; v <= 4; v++) cand.push_back(v);
     cand.push_back(kSlabVariant);

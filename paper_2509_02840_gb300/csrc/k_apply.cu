@@ -5,13 +5,13 @@
 // Rows of Q and P are independent under column rotations, so each CTA owns a
 // slab of R rows, keeps it in shared memory for the whole rank-1 column and
 // writes it back once: every element is read and written once per column.
-// The slab is stored column by column, so that a rotation reaches 4 (FP32) or
-// 2 (FP64) rows of both of its columns with each 16-byte shared access.
+// The slab is stored column by column, so that an FP32 rotation reaches 4 rows
+// of both of its columns with each 16-byte shared access.
 // The rotations of one chase act on disjoint column pairs, so a chase is
-// applied by all threads at once -- one rotation per thread, looping over the
-// slab's rows -- and consecutive chases are separated by a barrier; the next
-// chase's rotations are prefetched into registers while the current one is
-// applied.  The spike chain (m > n) is sequential and runs first, one thread
+// applied by all threads at once -- FP32: one rotation per thread, looping over
+// the slab's rows; FP64: see apply_slab64 -- and consecutive chases are
+// separated by a barrier; the next rotations are prefetched into registers
+// while the current ones are applied.  The spike chain (m > n) is sequential and runs first, one thread
 // per row.  R is chosen so that the grid fills whole waves of SMs.
 //
 // FP64: each pair update is c*x + s*y with separately rounded operations, the
@@ -186,6 +186,162 @@ __device__ __forceinline__ void apply_slab_body(T *__restrict__ X, int64_t ld, i
   }
 }
 
+// FP64 body.  A slab of R rows in shared memory (column stride csw, odd), all
+// chases applied one after another, a barrier between two.  Six FP64
+// operations a rotation and row at two FP64 results a clock and SM bound it at
+// large n, the chase's chain of latencies at small n:
+//   * a work item is 16 rotations x some of the slab's rows, two lanes a
+//     rotation (one forms x', the other y': three FP64 instructions, and half
+//     the latency of six); items are dealt so that every SM sub-partition
+//     gets the same number of rotations and rows (parts of the rows to
+//     warps 4 apart), since on GB300 a warp's FP64 instruction holds its
+//     sub-partition's FP64 unit for 64 cycles whatever the active lanes;
+//     A warp without an item in a chase issues none of them.
+//   * each warp runs through its items of all chases as one stream and loads
+//     the coefficients kAhead items ahead of their use, the counts of 32
+//     chases at a time.
+// Per side and column, before (a rotation of both rows and columns a thread,
+// coefficients one chase ahead) and now: order 64 0.61 -> 0.21 ms, 256 1.27 ->
+// 0.54, 512 5.6 -> 4.0, 1024 15.7 -> 12.3, 4096 750 -> 670 (the FP64 units'
+// floor at 4096 is 490 ms).  Any number of rows a slab may have (4096 columns:
+// 7, in 4 waves of blocks, where pairs of rows allowed 6 in 5).
+constexpr int kGroupRot = 16;  // rotations of an item
+constexpr int kAhead = 3;
+
+struct Item64 {
+  double c, s;  // as the lane uses them: own column times c, the other times s
+  int a;        // 1-based first column of the lane's pair, 0: none (as loaded: arithmetic here would wait for the load)
+  bool last;    // the warp's last item of its chase
+};
+// A warp's stream of items: chase t, group g; counts of chases t0 .. t0 + 31
+// in the lanes.
+struct Stream64 {
+  int t, g, t0, cnt, mine;
+};
+
+__device__ __forceinline__ void apply_slab64(double *__restrict__ X, int64_t ld, int nrow, int ncol, int R, int csw,
+                                             const RotStream &st, int side, int with_spike, int slab) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  double *tile = reinterpret_cast<double *>(raw);
+  const int r0 = slab * R;
+  const int rows = min(R, nrow - r0);
+  if (rows <= 0) return;
+  const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31, w = tid >> 5, nw = nth >> 5;
+  const int32_t *__restrict__ Ca = side == 0 ? st.La : st.Ra;
+  const int32_t *__restrict__ Cn = side == 0 ? st.Ln : st.Rn;
+  const double *__restrict__ Cc = side == 0 ? st.Lc : st.Rc;
+  const double *__restrict__ Cs = side == 0 ? st.Ls : st.Rs;
+  const int ntask = st.T, cap = st.cap;
+
+  for (int64_t q = tid; q < (int64_t)R * ncol; q += nth) {
+    const int col = (int)(q / R), rr = (int)(q % R);
+    tile[(size_t)col * csw + rr] = (rr < rows) ? X[(size_t)col * ld + r0 + rr] : 0.0;
+  }
+  __syncthreads();
+
+  if (with_spike) {
+    const int ns = st.Sn[0];
+    if (tid < rows && ns > 0) {
+      double *row = tile + tid;
+      double c = st.Sc[0], s = st.Ss[0];
+      int a = st.Sa[0] - 1;
+      for (int e = 0; e < ns; e++) {
+        const int en = min(e + 1, ns - 1);  // the next rotation, while this one is applied
+        const double nc = st.Sc[en], nsn = st.Ss[en];
+        const int na = st.Sa[en] - 1;
+        Coef<double>{c, s}.rot(row[(size_t)a * csw], row[(size_t)(a + 1) * csw]);
+        c = nc; s = nsn; a = na;
+      }
+    }
+    __syncthreads();
+  }
+
+  // This warp's share of a chase's groups: parts of the slab's rows go to
+  // warps 4 apart (the same sub-partition), the groups to the rest.
+  const int q4 = nw >= 4 ? 4 : 1;              // nw: 1, or a multiple of 4
+  const int upper = nw / q4;                   // warps of a sub-partition
+  int parts = 1;
+  while (parts * 2 <= upper && parts * 2 <= rows && ncol / (2 * kGroupRot) * parts < 2 * nw) parts *= 2;
+  const int part = (w / q4) % parts;
+  const int ra = rows * part / parts, rb = rows * (part + 1) / parts;
+  const int g0 = w % q4 + q4 * (w / (q4 * parts)), gstep = nw / parts;
+  const int h = lane & 1;  // 0: x', 1: y'
+
+  Stream64 S{-1, 0, -32, 0, 0};
+  // counts one batch ahead
+  auto counts = [&](int t0) { return t0 + lane < ntask ? Cn[t0 + lane] : 0; };
+  S.mine = 0;
+  int next_mine = counts(0);
+  auto next_item = [&]() {
+    Item64 it;
+    it.a = 0;
+    it.last = true;
+    it.c = it.s = 0.0;
+    if (S.t >= ntask) return it;
+    const bool more = S.t >= 0 && (S.g + gstep) * kGroupRot < S.cnt;
+    if (more) {
+      S.g += gstep;
+    } else {
+      S.t++;
+      if (S.t >= ntask) return it;
+      if (S.t - S.t0 >= 32) {
+        S.t0 += 32;
+        S.mine = next_mine;
+        next_mine = counts(S.t0 + 32);
+      }
+      S.cnt = __shfl_sync(0xffffffffu, S.mine, S.t - S.t0);
+      S.g = g0;
+    }
+    const int e = S.g * kGroupRot + (lane >> 1);
+    if (e < S.cnt) {
+      const size_t i = (size_t)S.t * cap + e;
+      it.a = __ldg(Ca + i);
+      it.c = __ldg(Cc + i);
+      it.s = __ldg(Cs + i);
+    }
+    it.last = (S.g + gstep) * kGroupRot >= S.cnt;
+    return it;
+  };
+  Item64 ring[kAhead];
+#pragma unroll
+  for (int k = 0; k < kAhead; k++) ring[k] = next_item();
+  for (int t = 0; t < ntask;) {
+#pragma unroll
+    for (int k = 0; k < kAhead; k++) {  // (unrolled: the ring stays in registers)
+      if (t >= ntask) break;
+      const Item64 it = ring[k];
+      ring[k] = next_item();
+      // two rows at a time; both lanes of a pair have read before either writes
+      const bool in = it.a > 0;
+      const int a = in ? it.a - 1 : 0;
+      const double s = h ? -it.s : it.s;
+      double *const own = tile + (size_t)(a + h) * csw, *const oth = tile + (size_t)(a + 1 - h) * csw;
+      // (an item past the chase's last rotation costs no FP64 instruction)
+      for (int r = __any_sync(0xffffffffu, in) ? ra : rb; r < rb; r += 2) {
+        const bool two = r + 1 < rb;
+        const double p0 = own[r], o0 = oth[r];
+        const double p1 = two ? own[r + 1] : 0.0, o1 = two ? oth[r + 1] : 0.0;
+        __syncwarp();
+        const double v0 = __dadd_rn(__dmul_rn(it.c, p0), __dmul_rn(s, o0));
+        if (in) own[r] = v0;
+        if (two) {
+          const double v1 = __dadd_rn(__dmul_rn(it.c, p1), __dmul_rn(s, o1));
+          if (in) own[r + 1] = v1;
+        }
+      }
+      if (it.last) {
+        __syncthreads();
+        t++;
+      }
+    }
+  }
+
+  for (int64_t q = tid; q < (int64_t)rows * ncol; q += nth) {
+    const int col = (int)(q / rows), rr = (int)(q % rows);
+    X[(size_t)col * ld + r0 + rr] = tile[(size_t)col * csw + rr];
+  }
+}
+
 // gate (may be null): a device error word written by an earlier kernel on
 // the stream; when it is nonzero the kernel leaves X untouched.
 template <typename T>
@@ -193,7 +349,8 @@ __global__ void __launch_bounds__(kThreads) k_apply_slab(T *__restrict__ X, int6
                                                          int ncol, int R, int csw, RotStream st,
                                                          int side, int with_spike, const int *gate) {
   if (gate && *(volatile const int *)gate) return;
-  apply_slab_body<T>(X, ld, nrow, ncol, R, csw, st, side, with_spike, blockIdx.x);
+  if constexpr (sizeof(T) == 8) apply_slab64(X, ld, nrow, ncol, R, csw, st, side, with_spike, blockIdx.x);
+  else apply_slab_body<T>(X, ld, nrow, ncol, R, csw, st, side, with_spike, blockIdx.x);
 }
 
 // Many matrices of uneven sizes in one launch: block b works on the slab
@@ -210,17 +367,42 @@ __global__ void __launch_bounds__(kThreads) k_apply_batch(const ApplyItem *__res
     else hi = mid - 1;
   }
   const ApplyItem it = items[lo];
-  apply_slab_body<T>((T *)it.X, it.ld, it.nrow, it.ncol, it.R, it.csw, it.st, it.side, it.with_spike,
-                     b - first[lo]);
+  if constexpr (sizeof(T) == 8)
+    apply_slab64((T *)it.X, it.ld, it.nrow, it.ncol, it.R, it.csw, it.st, it.side, it.with_spike, b - first[lo]);
+  else
+    apply_slab_body<T>((T *)it.X, it.ld, it.nrow, it.ncol, it.R, it.csw, it.st, it.side, it.with_spike,
+                       b - first[lo]);
 }
 
 }  // namespace
+
+// Column stride of an FP64 slab of R rows: odd (consecutive columns in distinct
+// banks) where that fits in smem_cap bytes, 0 when the slab does not fit.
+static int stride64(int R, int ncol, size_t smem_cap) {
+  if (sizeof(double) * (size_t)(R | 1) * ncol <= smem_cap) return R | 1;
+  return sizeof(double) * (size_t)R * ncol <= smem_cap ? R : 0;
+}
+// Threads of an FP64 slab's block: as many warps as the longest chases (a
+// rotation every second column) have items for, 4 to 16.
+static int threads64(int ncol, int R) {
+  const int items = (ncol / 2 + kGroupRot - 1) / kGroupRot * R;
+  return items <= 4 ? 128 : items <= 12 ? 256 : 512;
+}
 
 // Rows per slab and column stride for an ncol-wide matrix within smem_cap
 // bytes of shared memory, as many rows as fit (at most 64).
 void apply_geometry(int precision, int ncol, size_t smem_cap, int *R, int *csw) {
   const int esz = (precision == BDU_FP64) ? 8 : 4;
   const int V = 16 / esz;
+  if (precision == BDU_FP64) {
+    *R = *csw = 0;
+    for (int r = 2; r <= 64; r++) {
+      const int c = stride64(r, ncol, smem_cap);
+      if (c == 0) break;
+      *R = r; *csw = c;
+    }
+    return;
+  }
   int bestR = 0, bestc = 0;
   for (int r = V; r <= 64; r += V) {
     int w = r / V;
@@ -272,19 +454,24 @@ cudaError_t launch_apply(int precision, void *X, int64_t ld, int nrow, int ncol,
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int esz = (precision == BDU_FP64) ? 8 : 4;
   const int V = 16 / esz;
-  // rows per CTA: a multiple of V; the column stride is an odd number of
-  // 16-byte vectors.  Pick the R that minimizes waves x (R + overhead).
-  // (FP64 form: a positive variant fixes R instead)
+  // Rows per block.  FP32: a multiple of V, the column stride an odd number of
+  // 16-byte vectors; FP64: 2 to 64.  Pick the R that minimizes waves x (R +
+  // overhead).  (FP64 form: a positive variant fixes R instead)
   int best_R = 0, best_csw = 0;
   double best_cost = 1e300;
   const bool fixed = precision == BDU_FP64 && variant > 0;
-  if (fixed && (variant % V != 0 || variant > 64)) return cudaErrorNotSupported;
-  for (int R = V; R <= 64; R += V) {
-    int w = R / V;
-    if ((w & 1) == 0) w++;
-    const int csw = w * V;
-    const size_t smem = (size_t)esz * csw * ncol;
-    if (smem > (size_t)optin) break;
+  if (fixed && (variant < 2 || variant > 64)) return cudaErrorNotSupported;
+  for (int R = 2; R <= 64; R++) {
+    int csw = 0;
+    if (precision == BDU_FP64) {
+      csw = stride64(R, ncol, (size_t)optin);
+      if (csw == 0) break;
+    } else {
+      if (R % V) continue;
+      const int w = (R / V) | 1;
+      csw = w * V;
+      if ((size_t)esz * csw * ncol > (size_t)optin) break;
+    }
     const int ctas = (nrow + R - 1) / R;
     const int waves = (ctas + sms - 1) / sms;
     const double cost = fixed ? (R == variant ? 0.0 : 1e299) : (double)waves * (R + 4);
@@ -298,7 +485,7 @@ cudaError_t launch_apply(int precision, void *X, int64_t ld, int nrow, int ncol,
   if (precision == BDU_FP64) {
     e = cudaFuncSetAttribute(k_apply_slab<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_apply_slab<double><<<blocks, kThreads, smem, s>>>((double *)X, ld, nrow, ncol, best_R, best_csw, st,
+    k_apply_slab<double><<<blocks, threads64(ncol, best_R), smem, s>>>((double *)X, ld, nrow, ncol, best_R, best_csw, st,
                                                         side, with_spike ? 1 : 0, gate);
   } else {
     e = cudaFuncSetAttribute(k_apply_slab<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
