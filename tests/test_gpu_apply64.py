@@ -14,6 +14,8 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("nb", [0, 2, 6, 8, 64])
 @pytest.mark.parametrize("m,n", [(2, 2), (31, 31), (33, 32), (66, 34), (129, 128), (260, 259), (700, 40)])
 def test_items_and_slabs(m, n, nb):
+    if nb * m * 8 > 227 * 1024:
+        pytest.skip("a slab of nb rows does not fit in shared memory: the update refuses nb, as documented")
     Q, d, e, P = I.factorization(m, n, config=0, which=13 * m + n)
     B, C = I.dense_update(m, n, h=1, config=0)
     with bdu.Factorization(Q, d, e, P, precision=bdu.FP64, nb=nb) as F:
