@@ -1093,6 +1093,19 @@ bool alloc_records(bdu_ctx *h, RotStream &r, int T, int cap, int64_t m, bool mix
   return ok;
 }
 
+// Events of one call, destroyed at its end (which waits for nothing).
+struct EventPool {
+  std::vector<cudaEvent_t> all;
+  cudaEvent_t get() {
+    cudaEvent_t e = nullptr;
+    if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess) all.push_back(e);
+    return e;
+  }
+  ~EventPool() {
+    for (cudaEvent_t e : all) cudaEventDestroy(e);
+  }
+};
+
 struct BatchGuard {
   std::vector<bdu_ctx *> held;
   ~BatchGuard() {
@@ -1680,15 +1693,17 @@ static bdu_status update_batch_held(bdu_handle *hs, int count, const double *con
   if (ce == cudaSuccess) ce = launch_project_batch(precision, d_proj, (int)proj.size(), max_nrow, max_nrow, (int)max_r, s);
   if (ce != cudaSuccess) return cuda_fail(h0, ce, "batched projection");
 
-  int dev = 0, optin = 0;
+  int dev = 0, optin = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int esz = precision == BDU_FP64 ? 8 : 4;
+  EventPool events;
   for (int64_t k = 0; k < max_r; k++) {
     std::vector<ChaseArgs> chase;
     std::vector<const double *> cols, vcols;  // u columns (then v columns), in chase order
     std::vector<ApplyItem> apply;
-    std::vector<std::pair<bdu_ctx *, int>> tc_items;  // (handle, side) applied by the blocked apply
+    std::vector<std::pair<int, int>> tc_items;  // (item, side) applied by the blocked apply
     std::vector<int> first;
     int max_blocks = 0, slabs = 0;
     bool extra = false;  // some item's later projections are rotated inside its chase
@@ -1716,24 +1731,41 @@ static bdu_status update_batch_held(bdu_handle *hs, int count, const double *con
       for (int side = 0; side < 2; side++) {
         const int dim = side == 0 ? m : n;
         if (precision == BDU_MIXED && dim >= kBlockedFrom && h->st.tc_ws) {
-          tc_items.push_back({h, side});  // the blocked apply, as a single update takes it
+          tc_items.push_back({i, side});  // the blocked apply, as a single update takes it
           continue;
         }
         ApplyItem it{};
         it.X = side == 0 ? h->Q : h->P;
         it.ld = side == 0 ? m : n;
         it.nrow = it.ncol = side == 0 ? m : n;
-        apply_geometry(precision, it.ncol, (size_t)optin, &it.R, &it.csw);
+        apply_geometry(precision, it.ncol, (size_t)optin, 64, &it.R, &it.csw);
         if (it.R == 0) return fail(h, BDU_EINVAL, "matrix too wide for the batched apply");
         it.side = side;
         it.with_spike = (side == 0 && m > n) ? 1 : 0;
         it.st = h->st;
-        first.push_back(slabs);
-        slabs += (it.nrow + it.R - 1) / it.R;
-        const size_t sm = (size_t)esz * it.csw * it.ncol;
-        if (sm > smem) smem = sm;
         apply.push_back(it);
       }
+    }
+    // Rows per slab: a slab of R rows works for about R n^2 rotations, so R
+    // falls with n^2 from 64, by the largest factor that leaves two slabs an
+    // SM (with as many rows as fit everywhere, the widest factors' few slabs
+    // outlasted the rest: a batch of 16 FP64 sessions of 64..1024 176 ->
+    // 163 ms).
+    const double span = 64.0 * 4096 * 4096;
+    for (double t = 64.0 * 64 * 64; t <= span; t *= 1.25) {
+      slabs = 0;
+      for (auto &it : apply) {
+        const double rr = (double)it.st.cap * it.st.cap * 4;  // (cap: half the order of the middle matrix)
+        apply_geometry(precision, it.ncol, (size_t)optin, (int)std::min(64.0, t / rr), &it.R, &it.csw);
+        slabs += (it.nrow + it.R - 1) / it.R;
+      }
+      if (slabs <= 2 * sms) break;
+    }
+    slabs = 0;
+    for (auto &it : apply) {
+      first.push_back(slabs);
+      slabs += (it.nrow + it.R - 1) / it.R;
+      smem = std::max(smem, (size_t)esz * it.csw * it.ncol);
     }
     const int nact = (int)chase.size();
     cols.insert(cols.end(), vcols.begin(), vcols.end());
@@ -1744,32 +1776,63 @@ static bdu_status update_batch_held(bdu_handle *hs, int count, const double *con
     if (ce == cudaSuccess) ce = cudaMemcpyAsync(d_first, first.data(), sizeof(int) * first.size(), cudaMemcpyHostToDevice, s);
     if (ce == cudaSuccess) ce = launch_stage_batch(d_chase, d_cols, d_cols + nact, nact, s);
     if (ce == cudaSuccess) ce = launch_chase_batch(d_chase, nact, max_blocks, precision == BDU_MIXED, extra, s);
-    // mixed form: each item's later projections, rotated by this round's rotations
-    for (int i = 0; i < count && ce == cudaSuccess; i++) {
+    // Each item's own launches -- the mixed form's later projections, rotated
+    // by this round's rotations, the blocked applies, re-orthogonalizations --
+    // are grids of a few blocks: they go to the item's own stream, beside the
+    // other items' and the batched apply (one after the other on the batch's
+    // stream, 32 mixed sessions of 64..2048 took 231 ms a batch, now 171).  (An
+    // item's two blocked applies share
+    // a workspace, and its re-orthogonalization follows both kinds of apply.)
+    const bool own = precision == BDU_MIXED;
+    cudaEvent_t fork = nullptr, applied = nullptr;
+    if (own && ce == cudaSuccess) {
+      fork = events.get();
+      ce = cudaEventRecord(fork, s);
+    }
+    std::vector<char> described(count, 0);
+    for (int i = 0; own && i < count && ce == cudaSuccess; i++) {
       bdu_ctx *h = hs[i];
+      if (r[i] <= k) continue;
+      if (h->stream != s) ce = cudaStreamWaitEvent(h->stream, fork, 0);
       const int m = (int)h->m, n = (int)h->n, later = (int)(r[i] - k - 1);
-      if (later <= 0 || precision != BDU_MIXED || !rotate_vectors_supported(m, n)) continue;
-      ce = launch_chase_descriptors(h->st, 0, s);
-      if (ce == cudaSuccess) ce = launch_chase_descriptors(h->st, 1, s);
+      if (later <= 0 || !rotate_vectors_supported(m, n) || ce != cudaSuccess) continue;
+      ce = launch_chase_descriptors(h->st, 0, h->stream);
+      if (ce == cudaSuccess) ce = launch_chase_descriptors(h->st, 1, h->stream);
       if (ce == cudaSuccess)
         ce = launch_rotate_vector_sets(h->U + (k + 1) * m, h->U + (k + 1) * m, m, later, m, h->V + (k + 1) * n,
-                                       h->V + (k + 1) * n, n, later, n, h->st, m > n, h->status, s);
+                                       h->V + (k + 1) * n, n, later, n, h->st, m > n, h->status, h->stream);
+      described[i] = 1;
       h0->launches += 3;
     }
-    if (ce == cudaSuccess) ce = launch_apply_batch(precision, d_apply, d_first, (int)apply.size(), slabs, smem, s);
     for (size_t q = 0; q < tc_items.size() && ce == cudaSuccess; q++) {
-      bdu_ctx *h = tc_items[q].first;
-      const int side = tc_items[q].second, dim = side == 0 ? (int)h->m : (int)h->n;
+      const int i = tc_items[q].first, side = tc_items[q].second;
+      bdu_ctx *h = hs[i];
+      const int dim = side == 0 ? (int)h->m : (int)h->n;
       ce = launch_apply_tc((float *)(side == 0 ? h->Q : h->P), dim, dim, dim, h->st, side,
-                           side == 0 && h->m > h->n, h->status, false, 128, h->st.tc_ws, h->st.tc_ws_bytes, s);
+                           side == 0 && h->m > h->n, h->status, described[i], 128, h->st.tc_ws, h->st.tc_ws_bytes,
+                           h->stream);
+    }
+    if (ce == cudaSuccess) ce = launch_apply_batch(precision, d_apply, d_first, (int)apply.size(), slabs, smem, s);
+    h0->launches += 3;
+    if (own && ce == cudaSuccess) {
+      applied = events.get();
+      ce = cudaEventRecord(applied, s);
+    }
+    bdu_status rs = BDU_OK;
+    for (int i = 0; own && i < count; i++) {
+      bdu_ctx *h = hs[i];
+      if (r[i] <= k) continue;
+      if (h->stream != s && ce == cudaSuccess) ce = cudaStreamWaitEvent(h->stream, applied, 0);
+      if (ce == cudaSuccess && rs == BDU_OK) rs = reorth_after_column(h, h->stream);
+      if (h->stream == s) continue;
+      // (also after a failure: the batch's stream ends behind all of its work)
+      const cudaEvent_t join = events.get();
+      cudaError_t je = cudaEventRecord(join, h->stream);
+      if (je == cudaSuccess) je = cudaStreamWaitEvent(s, join, 0);
+      if (ce == cudaSuccess) ce = je;
     }
     if (ce != cudaSuccess) return cuda_fail(h0, ce, "batched update round");
-    h0->launches += 3;
-    for (int i = 0; i < count; i++)
-      if (r[i] > k) {
-        const bdu_status rs = reorth_after_column(hs[i], s);
-        if (rs != BDU_OK) return rs;
-      }
+    if (rs != BDU_OK) return rs;
   }
   h0->launches += 2;
   // each handle's later work waits for the batch

@@ -155,7 +155,7 @@ cudaError_t launch_apply(int precision, void *X, int64_t ld, int nrow, int ncol,
 
 cudaError_t launch_chase_batch(const ChaseArgs *d_items, int count, int max_blocks, int fast, bool extra,
                                cudaStream_t s);
-void apply_geometry(int precision, int ncol, size_t smem_cap, int *R, int *csw);
+void apply_geometry(int precision, int ncol, size_t smem_cap, int most, int *R, int *csw);
 cudaError_t launch_apply_reg(float *X, int64_t ld, int nrow, int ncol, const RotStream &st, int side,
                              bool with_spike, int *status, int sm_reserve, bool desc_ready, int layout,
                              cudaStream_t s);

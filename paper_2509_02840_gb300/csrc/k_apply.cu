@@ -18,6 +18,8 @@
 // same operations a one-rotation-at-a-time evaluation performs.  FP32 (the
 // mixed form): the generator's FP32 copies of (c, s) are applied with fused
 // multiply-adds.
+#include <algorithm>
+
 #include "bdu_internal.cuh"
 
 namespace bdu {
@@ -390,13 +392,14 @@ static int threads64(int ncol, int R) {
 }
 
 // Rows per slab and column stride for an ncol-wide matrix within smem_cap
-// bytes of shared memory, as many rows as fit (at most 64).
-void apply_geometry(int precision, int ncol, size_t smem_cap, int *R, int *csw) {
+// bytes of shared memory: as many rows as fit, at most `most` (and the least
+// there can be if that is fewer).
+void apply_geometry(int precision, int ncol, size_t smem_cap, int most, int *R, int *csw) {
   const int esz = (precision == BDU_FP64) ? 8 : 4;
   const int V = 16 / esz;
   if (precision == BDU_FP64) {
     *R = *csw = 0;
-    for (int r = 2; r <= 64; r++) {
+    for (int r = 2; r <= std::max(most, 2); r++) {
       const int c = stride64(r, ncol, smem_cap);
       if (c == 0) break;
       *R = r; *csw = c;
@@ -404,7 +407,7 @@ void apply_geometry(int precision, int ncol, size_t smem_cap, int *R, int *csw) 
     return;
   }
   int bestR = 0, bestc = 0;
-  for (int r = V; r <= 64; r += V) {
+  for (int r = V; r <= std::max(most, V); r += V) {
     int w = r / V;
     if ((w & 1) == 0) w++;
     const int c = w * V;
