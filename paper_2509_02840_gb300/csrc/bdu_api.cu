@@ -2054,31 +2054,35 @@ bdu_status bdu_singular_values(bdu_handle h, int64_t k, double *sv) {
   std::vector<double> d(n), e(n > 1 ? n - 1 : 1);
   cudaError_t ce = read_bidiagonal(h, d.data(), e.data());
   if (ce != cudaSuccess) return cuda_fail(h, ce, "bdu_singular_values");
-  // Golub-Kahan off-diagonal d_1, e_1, ..., d_n: squares, a Gershgorin bound
-  // of sigma_max and the smallest pivot magnitude
-  std::vector<double> b2(2 * n - 1);
-  double bmax2 = 0.0, hi = 0.0, prev = 0.0;
+  // Golub-Kahan off-diagonal d_1, e_1, ..., d_n: a Gershgorin bound of
+  // sigma_max, scaled into [1, 2) by a power of two, and the squares
+  double hi = 0.0, prev = 0.0;
   for (int64_t i = 0; i < 2 * n - 1; i++) {
     const double b = fabs((i & 1) ? e[i / 2] : d[i / 2]);
-    b2[i] = b * b;
-    bmax2 = b2[i] > bmax2 ? b2[i] : bmax2;
     hi = prev + b > hi ? prev + b : hi;
     prev = b;
   }
   hi = prev > hi ? prev : hi;
   hi = hi * (1.0 + 8.0 * DBL_EPSILON) + DBL_MIN;
-  const double pivmin = DBL_MIN * (bmax2 > 1.0 ? bmax2 : 1.0);
+  const int ex = std::isfinite(hi) ? ilogb(hi) : 0;
+  std::vector<double> b2(2 * n - 1);
+  for (int64_t i = 0; i < 2 * n - 1; i++) {
+    const double b = scalbn(fabs((i & 1) ? e[i / 2] : d[i / 2]), -ex);
+    b2[i] = b * b;
+  }
+  hi = scalbn(hi, -ex);
   const size_t bytes = sizeof(double) * (size_t)(2 * n - 1 + k) + 64;
   double *ws = (double *)dev_alloc(h, bytes);
   if (!ws) return fail(h, BDU_ENOMEM, "bdu_singular_values: workspace allocation failed");
   double *db2 = ws, *dsv = ws + (2 * n - 1);
   cudaStream_t s = h->stream;
   ce = cudaMemcpyAsync(db2, b2.data(), sizeof(double) * b2.size(), cudaMemcpyHostToDevice, s);
-  if (ce == cudaSuccess) ce = launch_bidiag_svals(db2, (int)n, hi, pivmin, (int)k, dsv, s);
+  if (ce == cudaSuccess) ce = launch_bidiag_svals(db2, (int)n, hi, (int)k, dsv, s);
   if (ce == cudaSuccess) ce = cudaMemcpyAsync(sv, dsv, sizeof(double) * k, cudaMemcpyDeviceToHost, s);
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
   dev_free(h, ws);
   if (ce != cudaSuccess) return cuda_fail(h, ce, "bdu_singular_values");
+  for (int64_t i = 0; i < k; i++) sv[i] = scalbn(sv[i], ex);
   h->launches += 1;
   return BDU_OK;
 }
