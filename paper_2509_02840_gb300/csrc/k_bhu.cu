@@ -154,8 +154,9 @@ __device__ bool grid_barrier(const BhuArgs &A, unsigned &gen) {
       }
     }
     // (the acquire load above orders this block's later reads after every
-    // block's writes, which each fenced before arriving)
-    if (*(volatile int *)A.status & ERR_BHU) stop = 1;
+    // block's writes, which each fenced before arriving; a block that has
+    // passed while another gave up stops at its next barrier, inside the wait:
+    // reading the status word here cost every barrier another L2 round trip)
     s_stop = stop;
   }
   __syncthreads();
