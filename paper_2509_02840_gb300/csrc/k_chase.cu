@@ -111,56 +111,13 @@ __device__ __forceinline__ float f32_of(double x) {
   return __uint_as_float(r | sign);
 }
 
-// Same rotation from y ~ 1/sqrt(f^2 + g^2): both inputs are scaled exactly by
-// the power of two that brings the larger into [0.5, 1), so q = f^2 + g^2 lies
-// in [0.25, 2); y0 = rsqrtf(q) (q truncated to FP32 and y0 widened back
-// through the bit patterns, about 22 correct bits) is refined by
-// y = y0 (1 + e/2 + 3e^2/8) with e = 1 - q y0^2 (third-order Newton step,
-// error about e^3).  Inputs outside [2^-1021, 2^1022), subnormal, or with a
-// ratio below 2^-1021 take the exact path.  Results are those of the same
-// formulas with the scalings done as FP64 multiplies (which are exact).
-__device__ __forceinline__ bool rotg_fast(double f, double g, double &c, double &s, double &r) {
-  const unsigned long long bf = absbits(f), bg = absbits(g);
-  const unsigned long long bm = bf > bg ? bf : bg, bn = bf > bg ? bg : bf;
-  const int ex = (int)(bm >> 52), en = (int)(bn >> 52);
-  // the exact path when the scalings below would leave the normal range: the
-  // larger input's exponent outside [2, 2044], or the smaller input subnormal
-  // or more than 2^1021 below the larger
-  if (bg != 0 && (ex < 2 || ex > 2044 || (bn != 0 && (en == 0 || en + 1021 < ex)))) return rotg_exact(f, g, c, s, r);
-  // fs = f 2^(1022-ex), gs = g 2^(1022-ex) and r = |r_s| 2^(ex-1022): exact
-  // power-of-two scalings, done on the exponent field (integer pipes)
-  const long long dk = (long long)(1022 - ex) << 52;
-  const double fs = bf == 0 ? 0.0 : __longlong_as_double(__double_as_longlong(f) + dk);
-  const double gs = bg == 0 ? 0.0 : __longlong_as_double(__double_as_longlong(g) + dk);
-  const double q = fma(fs, fs, gs * gs);
-  const unsigned qf = (unsigned)(((unsigned long long)__double_as_longlong(q) >> 29) - (896ULL << 23));
-  double y = __longlong_as_double((long long)(((unsigned long long)__float_as_uint(rsqrtf(__uint_as_float(qf))) << 29) +
-                                              (896ULL << 52)));
-  const double e = fma(-(q * y), y, 1.0);
-  y = fma(y * e, fma(0.375, e, 0.5), y);
-  const bool fz = bf == 0;
-  const long long sf = __double_as_longlong(f) & (long long)0x8000000000000000ULL;  // sign(f)
-  const double fa = __longlong_as_double((long long)absbits(fs));                  // |fs|
-  const double gsg = __longlong_as_double(__double_as_longlong(gs) ^ sf);          // sign(f) gs
-  const double qy = q * y;                                                         // |r| scaled, in [0.5, 1.5)
-  c = fz ? 0.0 : fa * y;
-  s = fz ? 1.0 : gsg * y;
-  r = fz ? g : __longlong_as_double((__double_as_longlong(qy) - dk) ^ sf);
-  return bg != 0;
-}
-
+// A pair (x, y) after the rotation.
 template <bool FAST> struct Arith;
 template <> struct Arith<false> {
-  static __device__ __forceinline__ bool rot(double f, double g, double &c, double &s, double &r) {
-    return rotg_exact(f, g, c, s, r);
-  }
   static __device__ __forceinline__ double px(double c, double s, double x, double y) { return add(mul(c, x), mul(s, y)); }
   static __device__ __forceinline__ double py(double c, double s, double x, double y) { return add(mul(-s, x), mul(c, y)); }
 };
 template <> struct Arith<true> {
-  static __device__ __forceinline__ bool rot(double f, double g, double &c, double &s, double &r) {
-    return rotg_fast(f, g, c, s, r);
-  }
   static __device__ __forceinline__ double px(double c, double s, double x, double y) { return fma(c, x, s * y); }
   static __device__ __forceinline__ double py(double c, double s, double x, double y) { return fma(c, y, -(s * x)); }
 };
@@ -310,8 +267,14 @@ __device__ __forceinline__ double rsqrt_f64(double q) {
 }
 
 // The rotation of one chase by its four lanes (f, g the same in all of them;
-// every lane of the warp calls it): rotg_fast / rotg_exact, bit for bit.  c
-// and s end up in every lane, r in lanes 2 and 3.
+// every lane of the warp calls it).  c and s end up in every lane, r in lanes
+// 2 and 3.
+//
+// Fast: from y ~ 1/sqrt(f^2 + g^2) of the inputs scaled by the power of two
+// that brings the larger into [0.5, 1) (exact, on the exponent fields; f^2 +
+// g^2 then lies in [0.25, 2)).  Inputs whose scaling would leave the normal
+// range -- the larger exponent outside [2, 2044], the smaller input subnormal
+// or more than 2^1021 below the larger -- take the plain form.
 //
 // Exact: the square root and the two quotients are formed from y ~
 // 1/sqrt(f^2 + g^2) by Newton corrections with exact remainders (Markstein,
@@ -319,11 +282,11 @@ __device__ __forceinline__ double rsqrt_f64(double q) {
 // the rounding interval around it through its exact remainder: h is the
 // rounded root of q iff q - h^2 lies in (-h ulp, h ulp], a quotient the
 // rounded one iff its remainder is below half an ulp of it times h (a tie
-// cannot occur).  18 FP64 instructions against the library's division and
-// square root at n = 1024: 1.7k cycles a step against 5.9k.  The scaling by
+// cannot occur).  18 FP64 instructions: the rotation took 4.4k cycles at n =
+// 1024 with the library's square root and division and takes 1.8k.  The scaling by
 // the larger exponent is exact and does not change any rounding while both
 // inputs lie within 2^-500..2^500 and within 2^900 of each other; for others
-// plain is set, and the caller takes the plain form (rot_plain).
+// plain is set, and the caller takes the plain form (rot_plain: rotg_exact).
 template <bool FAST>
 __device__ __forceinline__ void rot_lanes(double f, double g, int lane, double &c, double &s, double &r, bool &plain) {
   const int role = lane & 3;
@@ -377,10 +340,8 @@ __device__ __forceinline__ void rot_lanes(double f, double g, int lane, double &
   r = fz ? g : r;
 }
 
-template <bool FAST>
 __device__ __noinline__ void rot_plain(double f, double g, double &c, double &s, double &r) {
-  if (FAST) rotg_fast(f, g, c, s, r);
-  else rotg_exact(f, g, c, s, r);
+  rotg_exact(f, g, c, s, r);
 }
 
 // One op of a chase, as a lane sees it: byte offsets in the window of the
@@ -541,7 +502,7 @@ __device__ __forceinline__ void rotate_chases(const ChaseArgs &Ar, Shared &S, co
     // (scaling extremes; near row 1 the plan above does not hold)
     const bool top = __any_sync(0xffffffffu, least <= kNearTop);
     if (__any_sync(0xffffffffu, plain)) {
-      if (plain) rot_plain<FAST>(f, g, c, s, r);
+      if (plain) rot_plain(f, g, c, s, r);
     }
     const double nx = A::px(c, s, x, y), ny = A::py(c, s, x, y);
     if (FAST) {
@@ -797,7 +758,7 @@ __device__ __forceinline__ void run_spike(const ChaseArgs &Ar) {
       double c = 1.0, s = 0.0, r = 0.0;
       bool plain;
       rot_lanes<FAST>(f, run, lane, c, s, r, plain);
-      if (plain) rot_plain<FAST>(f, run, c, s, r);
+      if (plain) rot_plain(f, run, c, s, r);
       const bool ok = nz(run);
       r = __shfl_sync(0xffffffffu, r, 2);
       if (lane == k) {
