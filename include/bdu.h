@@ -112,10 +112,10 @@ typedef struct {
                          The capture runs on the handle's stream: work that other threads
                          enqueue on that stream during an update would be captured too. */
   int64_t step_budget; /* watchdog of the chase: steps (one rotation of each chase that may
-                         advance) a warp may take per rank-1 column before the kernel
-                         stops and the update fails with BDU_ETIMEOUT (poisoning the
-                         handle); 0 = 64 (n + 16) + 4096 (default; a column needs
-                         about 11 n in all) */
+                         advance) a warp may take for a group of 32 chases before the
+                         kernel stops and the update fails with BDU_ETIMEOUT
+                         (poisoning the handle); 0 = 64 (n + 16) + 4096 (default; a
+                         group needs up to about 1.3 n + 100) */
   int reorth_every;   /* BDU_MIXED: one Newton-Schulz re-orthogonalization step of Q (P)
                          behind the application of a factor's first rank-1 column and
                          then of every reorth_every-th (in the overlapped and rank-r
@@ -481,7 +481,7 @@ void bdu_thin_destroy(bdu_thin_handle h);
  *   BDU_INJECT_NONE: off (the default; value ignored);
  *   BDU_INJECT_STEP_BUDGET: a chase launched with no step budget of its own
  *     (bdu_options.step_budget = 0, and the allocation-free entry point) stops
- *     after `value` synchronous steps per rank-1 column;
+ *     after `value` steps of a warp on a group of chases;
  *   BDU_INJECT_APPLY_STALL: the FP32 register-resident rotation apply (mixed
  *     form) starts no copy of rotation records, and its compute warps give up
  *     after `value` polls of a wait;

@@ -98,7 +98,7 @@ struct ChaseArgs {
   int *sync;          // chase_sync_ints(m, n) ints, zero before the launch
   int nsync;          // (of a batch's item) that number, for the staging kernel to clear
   int blocks;         // thread blocks (set by launch_chase; of a batch's item, by the caller)
-  long long step_budget;  // bound on the steps of one warp per column; 0: 64 (n + 16) + 4096
+  long long step_budget;  // bound on the steps of one warp for a group; 0: 64 (n + 16) + 4096
 };
 
 // One matrix (Q or P of one factorization) for the batched apply.

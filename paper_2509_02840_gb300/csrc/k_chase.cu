@@ -816,11 +816,12 @@ __device__ __forceinline__ void engine(const ChaseArgs &Ar) {
     S.tab[e] = t;
   }
   if (me < kStates) S.info[me] = geo_info(me);
-  const int max_steps = (int)min(Ar.step_budget > 0 ? Ar.step_budget : 64LL * (n + 16) + 4096, 0x7ffffffeLL);
+  const long long budget = 64LL * (n + 16) + 4096;
+  const int max_steps = (int)min(Ar.step_budget > 0 ? Ar.step_budget : budget, 0x7ffffffeLL);
   // a poll takes tens of nanoseconds at least, a step half a microsecond; the
   // spike runs before everything else
-  const long long max_polls = 256LL * max_steps + 64LL * (m - n);
-  int steps = 0;
+  const long long max_polls = 256 * budget + 64LL * (m - n);
+  int steps = 0;  // of this warp, on the group at hand
   if (me == 0) S.far = kFar;
   for (;;) {
     __syncthreads();
@@ -831,6 +832,7 @@ __device__ __forceinline__ void engine(const ChaseArgs &Ar) {
     __syncthreads();
     const int s = S.ticket;
     if (s >= groups) return;
+    steps = 0;
     const int phase = s < F.g1 ? 1 : s < F.g1 + F.g2 ? 2 : 3;
     const int q0 = (s - (phase == 1 ? 0 : phase == 2 ? F.g1 : F.g1 + F.g2)) * kGroup;
     const int cnt = min(kGroup, (phase == 1 ? F.p1 : phase == 2 ? F.p2 : F.p3) - q0);

@@ -45,3 +45,19 @@ def test_chases_that_find_nothing_to_do():
     want = O.update(Q, d, e, P, b.reshape(-1, 1), c.reshape(-1, 1))
     for name, x, y in zip("QdeP", got, want):
         assert np.array_equal(x, y), name
+
+
+def test_one_block_takes_every_group_of_a_large_column():
+    """The watchdog bounds the steps of a group, not of the block that runs them all."""
+    n = 1700
+    Q = np.eye(n, order="F")
+    g = np.random.default_rng(8)
+    d, e = g.uniform(1, 10, n), g.standard_normal(n - 1)
+    b, c = g.standard_normal(n), g.standard_normal(n)
+    got = []
+    for engine in (0, 1):
+        with bdu.Factorization(Q, d, e, Q, precision=bdu.MIXED, engine=engine) as F:
+            F.update(b, c)
+            got.append(F.read())
+    for name, x, y in zip("QdeP", *got):
+        assert np.array_equal(x, y), name
