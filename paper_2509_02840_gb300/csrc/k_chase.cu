@@ -59,9 +59,12 @@
 #include <algorithm>
 
 #include "bdu_internal.cuh"
+#include "chase_schedule.cuh"
 
 namespace bdu {
 namespace {
+
+using namespace chase;
 
 // ----------------------------------------------------------------------------
 // rotation arithmetic
@@ -125,10 +128,6 @@ template <> struct Arith<true> {
 // ----------------------------------------------------------------------------
 // chases, groups, the window
 // ----------------------------------------------------------------------------
-constexpr int kLanes = 4;                    // lanes of a chase
-constexpr int kSlots = 32 / kLanes;          // chases of a warp
-constexpr int kRotWarps = 4;                 // warps that rotate (one per SM sub-partition)
-constexpr int kGroup = kRotWarps * kSlots;   // chases of a group
 constexpr int kThreads = 32 * (kRotWarps + 2);
 // Rows of the window.  A group's chases are at most 6 positions apart while
 // none of them has to wait for rows (lag 4, and a position advances by up to
@@ -143,40 +142,6 @@ constexpr int kPad = 8;                      // rows of zeros below the band
 constexpr int kFar = 1 << 29;                // a position or row beyond every other
 constexpr int kAborted = -1;                 // progress word of a group that gave up
 
-enum : int { S_L0 = 0, S_R1 = 1, S_L1 = 2, S_A = 3, S_B = 4, S_C = 5, S_CL = 6, S_CR = 7, S_P2 = 8 };
-constexpr int kStates = 9;
-
-// Geometry of each op kind.  An op at position a rotates rows (a, a+1) over
-// columns a-dl .. a-dl+w-1, or columns (a, a+1) over as many rows.  src 0: the
-// entry eliminated is the first pair's second, 1: u(a+1) against u(a), 2: row
-// 1's (1, a+1) against (1, a); S_R1 also rotates v(a), v(a+1).  next, dpos:
-// the op that follows while the bulge exists, and its distance; it exists
-// while a + loff <= N (limN) or <= n.
-struct Geo {
-  bool rows;
-  int dl, w, src;
-  bool withv;
-  int next, dpos;
-  bool limN;
-  int loff;
-};
-__host__ __device__ constexpr Geo geo_of(int st) {
-  return st == S_L0 ? Geo{true, 0, 3, 1, false, S_R1, 1, false, 2}
-       : st == S_R1 ? Geo{false, 1, 4, 0, true, S_L1, 1, true, 2}
-       : st == S_L1 ? Geo{true, 1, 4, 0, false, S_R1, 1, false, 2}
-       : st == S_A  ? Geo{true, 0, 4, 0, false, S_B, 2, false, 3}
-       : st == S_B  ? Geo{false, 2, 5, 0, false, S_CL, 1, true, 2}
-       : st == S_C  ? Geo{false, 1, 4, 0, false, S_CL, 1, true, 2}
-       : st == S_CL ? Geo{true, 1, 5, 0, false, S_CR, 2, false, 3}
-       : st == S_CR ? Geo{false, 2, 5, 0, false, S_CL, 1, true, 2}
-       :              Geo{false, 1, 4, 2, false, S_CL, 1, true, 2};  // S_P2
-}
-// Number of pairs rotated besides the source pair, and which of them holds the
-// bulge (its first cell is the entry the chase looks at next).
-__host__ __device__ constexpr int geo_pairs(int st) {
-  return geo_of(st).w - (geo_of(st).src == 0 ? 1 : 0) + (geo_of(st).withv ? 1 : 0);
-}
-__host__ __device__ constexpr int geo_bulge(int st) { return geo_pairs(st) - 1 - (geo_of(st).withv ? 1 : 0); }
 // info word of a state: bit 0 rows, 1-2 bulge pair, 3-6 next, 7-8 dpos,
 // 9 limN, 10-12 loff, 13 the chase ends when this op finds nothing to rotate
 __host__ __device__ constexpr int geo_info(int st) {
@@ -186,31 +151,6 @@ __host__ __device__ constexpr int geo_info(int st) {
 // Byte offset of cell `cell` of the row `drow` away from the position, from
 // the row two above it (the topmost an op touches).
 __device__ __forceinline__ int rel(int drow, int cell) { return (drow + 2) * kRowBytes + cell * 8; }
-
-// The problem as a sequence of groups: phases 1, 2 and 3 in groups of kGroup
-// chases (no group crosses a phase; phase 1 has one even without chases, since
-// its last group does the fold).
-__host__ __device__ inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
-struct Phases {
-  int N, p1, p2, p3, g1, g2, g3;
-};
-__host__ __device__ inline Phases phases_of(int m, int n) {
-  Phases f;
-  f.N = m > n ? n + 1 : n;
-  f.p1 = f.N - 1;
-  f.p2 = n > 2 ? n - 2 : 0;
-  f.p3 = 2 * (f.N == n + 1 ? n : n - 1);
-  f.g1 = f.p1 > 0 ? ceil_div(f.p1, kGroup) : 1;
-  f.g2 = ceil_div(f.p2, kGroup);
-  f.g3 = ceil_div(f.p3, kGroup);
-  return f;
-}
-// First op (state, position) of chase q (0-based) of a phase.
-__device__ __forceinline__ void first_op(const Phases &F, int n, int phase, int q, int &st, int &pos) {
-  if (phase == 1) { st = S_L0; pos = F.N - q - 1; }
-  else if (phase == 2) { st = S_P2; pos = n - q - 1; }
-  else { st = (q & 1) ? S_C : S_A; pos = q / 2 + 1 + (q & 1); }
-}
 
 // progress words in shared memory (one CTA) and in global memory (the groups)
 __device__ __forceinline__ int ld_cta(const int *p) {
@@ -399,9 +339,10 @@ __device__ __forceinline__ void rotate_chases(const ChaseArgs &Ar, Shared &S, co
   using A = Arith<FAST>;
   const int lane = threadIdx.x & 31, q = lane & 3, slot = w * kSlots + (lane >> 2);
   const int n = Ar.n, N = F.N;
-  bool done = slot >= cnt;
   int st = S_A, pos = kFar;
-  if (!done) first_op(F, n, phase, q0 + slot, st, pos);
+  const bool mine = slot < cnt;
+  bool done = !mine || !first_op(F, n, phase, q0 + slot, st, pos);
+  if (done) pos = kFar;
   int eff = done ? 0 : pos;  // what the next chase stays behind
   // a finished chase passes on what it had to stay behind itself
   auto relay = [](int ahead) { return ahead >= kFar ? kFar : ahead - 1; };
@@ -411,6 +352,7 @@ __device__ __forceinline__ void rotate_chases(const ChaseArgs &Ar, Shared &S, co
   // where the lane writes its part of a record: the pair (lane 0), c (1), s (3)
   char *recL = nullptr, *recR = nullptr;
   const int stride = q == 0 ? 4 : 8;
+  if (mine && done && q == 0) Ar.st.Ln[t] = Ar.st.Rn[t] = 0;
   if (!done) {
     const size_t rec = (size_t)t * cap;
     if (q == 0) {
@@ -847,8 +789,7 @@ __device__ __forceinline__ void engine(const ChaseArgs &Ar) {
       int least = kFar;
       for (int k = me * kSlots; k < min(cnt, (me + 1) * kSlots); k++) {
         int a, p;
-        first_op(F, n, phase, q0 + k, a, p);
-        least = min(least, p);
+        if (first_op(F, n, phase, q0 + k, a, p)) least = min(least, p);
       }
       S.least[me] = least;
     }
