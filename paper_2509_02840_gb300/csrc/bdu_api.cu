@@ -283,7 +283,7 @@ bdu_status check_device_status(bdu_ctx *h) {
   if (st & ERR_ROTVEC) return fail(h, BDU_ETIMEOUT, "a bounded wait of the vector rotation ran out");
   if (st & ERR_GEMM) return fail(h, BDU_ETIMEOUT, "a bounded wait of the re-orthogonalization GEMM ran out");
   if (st & ERR_BHU) return fail(h, BDU_ETIMEOUT, "a grid barrier of the BHU kernel ran out");
-  if (st & ERR_RANGE) return fail(h, BDU_EINTERNAL, "a rotation record named a pair outside the vector");
+  if (st & ERR_RANGE) return fail(h, BDU_EINTERNAL, "a rotation record named a pair outside the vector or factor");
   if (st) return fail(h, BDU_EINTERNAL, "device invariant check failed (status bits 0x%x)", st);
   return BDU_OK;
 }
@@ -1743,6 +1743,7 @@ static bdu_status update_batch_held(bdu_handle *hs, int count, const double *con
         it.side = side;
         it.with_spike = (side == 0 && m > n) ? 1 : 0;
         it.st = h->st;
+        it.status = h->status;
         apply.push_back(it);
       }
     }

@@ -15,7 +15,7 @@ enum : int {
   ERR_SCHEDULE = 8,  // an op found a zero where the schedule guarantees a nonzero
   ERR_APPLY = 16,    // a bounded wait of the register-resident apply ran out
   ERR_ROTVEC = 32,   // a bounded wait of the vector rotation ran out
-  ERR_RANGE = 64,    // a record named a pair outside the vector (skipped)
+  ERR_RANGE = 64,    // a record named a pair outside the vector or factor (skipped)
   ERR_GEMM = 128,    // a bounded wait of the tensor-core GEMM ran out
   ERR_BHU = 256,     // a grid barrier of the BHU kernel ran out
 };
@@ -107,6 +107,7 @@ struct ApplyItem {
   int64_t ld;
   int nrow, ncol, R, csw, side, with_spike;
   RotStream st;
+  int *status;  // device error word (ERR_RANGE)
 };
 
 // One projection X^T B for the batched projection.

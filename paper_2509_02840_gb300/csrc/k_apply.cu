@@ -18,6 +18,9 @@
 // same operations a one-rotation-at-a-time evaluation performs.  FP32 (the
 // mixed form): the generator's FP32 copies of (c, s) are applied with fused
 // multiply-adds.
+//
+// The slab is indexed with the columns that the records name, so a record whose
+// pair lies outside the matrix is skipped and reported (ERR_RANGE).
 #include <algorithm>
 
 #include "bdu_internal.cuh"
@@ -86,7 +89,7 @@ template <> struct Vec<double> {
 template <typename T>
 __device__ __forceinline__ void apply_slab_body(T *__restrict__ X, int64_t ld, int nrow, int ncol, int R,
                                                 int csw, const RotStream &st, int side, int with_spike,
-                                                int slab) {
+                                                int slab, int *status) {
   using VT = typename Vec<T>::type;
   constexpr int V = Vec<T>::V;
   extern __shared__ __align__(16) unsigned char raw[];
@@ -149,7 +152,7 @@ __device__ __forceinline__ void apply_slab_body(T *__restrict__ X, int64_t ld, i
     // apply chase t: each owned rotation to all rows of the slab, V rows per access
 #pragma unroll
     for (int k = 0; k < kPer; k++) {
-      if (ca[k] >= 0) {
+      if ((unsigned)ca[k] < (unsigned)(ncol - 1)) {
         VT *pa = reinterpret_cast<VT *>(tile + (size_t)ca[k] * csw);
         VT *pb = reinterpret_cast<VT *>(tile + (size_t)(ca[k] + 1) * csw);
         for (int q = 0; q < nv; q++) {
@@ -158,6 +161,8 @@ __device__ __forceinline__ void apply_slab_body(T *__restrict__ X, int64_t ld, i
           pa[q] = x;
           pb[q] = y;
         }
+      } else if (ca[k] != -1 && status) {
+        atomicOr(status, ERR_RANGE);
       }
     }
     // chases longer than the register-held part
@@ -165,8 +170,13 @@ __device__ __forceinline__ void apply_slab_body(T *__restrict__ X, int64_t ld, i
     for (int e = tid + kPer * kThreads; e < ccnt; e += kThreads) {
       const size_t i = (size_t)t * cap + e;
       const Coef<T> k = Coef<T>::load(st, side, i);
-      VT *pa = reinterpret_cast<VT *>(tile + (size_t)(Ca[i] - 1) * csw);
-      VT *pb = reinterpret_cast<VT *>(tile + (size_t)Ca[i] * csw);
+      const int a = Ca[i] - 1;
+      if ((unsigned)a >= (unsigned)(ncol - 1)) {
+        if (status) atomicOr(status, ERR_RANGE);
+        continue;
+      }
+      VT *pa = reinterpret_cast<VT *>(tile + (size_t)a * csw);
+      VT *pb = reinterpret_cast<VT *>(tile + (size_t)(a + 1) * csw);
       for (int q = 0; q < nv; q++) {
         VT x = pa[q], y = pb[q];
         Vec<T>::rot(k, x, y);
@@ -222,7 +232,7 @@ struct Stream64 {
 };
 
 __device__ __forceinline__ void apply_slab64(double *__restrict__ X, int64_t ld, int nrow, int ncol, int R, int csw,
-                                             const RotStream &st, int side, int with_spike, int slab) {
+                                             const RotStream &st, int side, int with_spike, int slab, int *status) {
   extern __shared__ __align__(16) unsigned char raw[];
   double *tile = reinterpret_cast<double *>(raw);
   const int r0 = slab * R;
@@ -314,7 +324,8 @@ __device__ __forceinline__ void apply_slab64(double *__restrict__ X, int64_t ld,
       const Item64 it = ring[k];
       ring[k] = next_item();
       // two rows at a time; both lanes of a pair have read before either writes
-      const bool in = it.a > 0;
+      const bool in = (unsigned)(it.a - 1) < (unsigned)(ncol - 1);
+      if (it.a != 0 && !in && status) atomicOr(status, ERR_RANGE);
       const int a = in ? it.a - 1 : 0;
       const double s = h ? -it.s : it.s;
       double *const own = tile + (size_t)(a + h) * csw, *const oth = tile + (size_t)(a + 1 - h) * csw;
@@ -349,10 +360,10 @@ __device__ __forceinline__ void apply_slab64(double *__restrict__ X, int64_t ld,
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_apply_slab(T *__restrict__ X, int64_t ld, int nrow,
                                                          int ncol, int R, int csw, RotStream st,
-                                                         int side, int with_spike, const int *gate) {
+                                                         int side, int with_spike, int *status, const int *gate) {
   if (gate && *(volatile const int *)gate) return;
-  if constexpr (sizeof(T) == 8) apply_slab64(X, ld, nrow, ncol, R, csw, st, side, with_spike, blockIdx.x);
-  else apply_slab_body<T>(X, ld, nrow, ncol, R, csw, st, side, with_spike, blockIdx.x);
+  if constexpr (sizeof(T) == 8) apply_slab64(X, ld, nrow, ncol, R, csw, st, side, with_spike, blockIdx.x, status);
+  else apply_slab_body<T>(X, ld, nrow, ncol, R, csw, st, side, with_spike, blockIdx.x, status);
 }
 
 // Many matrices of uneven sizes in one launch: block b works on the slab
@@ -370,10 +381,11 @@ __global__ void __launch_bounds__(kThreads) k_apply_batch(const ApplyItem *__res
   }
   const ApplyItem it = items[lo];
   if constexpr (sizeof(T) == 8)
-    apply_slab64((T *)it.X, it.ld, it.nrow, it.ncol, it.R, it.csw, it.st, it.side, it.with_spike, b - first[lo]);
+    apply_slab64((T *)it.X, it.ld, it.nrow, it.ncol, it.R, it.csw, it.st, it.side, it.with_spike, b - first[lo],
+                 it.status);
   else
     apply_slab_body<T>((T *)it.X, it.ld, it.nrow, it.ncol, it.R, it.csw, it.st, it.side, it.with_spike,
-                       b - first[lo]);
+                       b - first[lo], it.status);
 }
 
 }  // namespace
@@ -489,12 +501,12 @@ cudaError_t launch_apply(int precision, void *X, int64_t ld, int nrow, int ncol,
     e = cudaFuncSetAttribute(k_apply_slab<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     k_apply_slab<double><<<blocks, threads64(ncol, best_R), smem, s>>>((double *)X, ld, nrow, ncol, best_R, best_csw, st,
-                                                        side, with_spike ? 1 : 0, gate);
+                                                        side, with_spike ? 1 : 0, status, gate);
   } else {
     e = cudaFuncSetAttribute(k_apply_slab<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     k_apply_slab<float><<<blocks, kThreads, smem, s>>>((float *)X, ld, nrow, ncol, best_R, best_csw, st,
-                                                       side, with_spike ? 1 : 0, gate);
+                                                       side, with_spike ? 1 : 0, status, gate);
   }
   return cudaGetLastError();
 }
