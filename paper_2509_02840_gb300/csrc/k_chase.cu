@@ -152,7 +152,11 @@ __host__ __device__ constexpr int geo_info(int st) {
 // the row two above it (the topmost an op touches).
 __device__ __forceinline__ int rel(int drow, int cell) { return (drow + 2) * kRowBytes + cell * 8; }
 
-// progress words in shared memory (one CTA) and in global memory (the groups)
+// Progress words in shared memory (one CTA) and in global memory (the groups).
+// Lane 0's reading of a word counts for its warp: the lanes of a chase decide
+// alike, and what the word's writer stored before it is seen by lane 0 at once
+// and by the others after the warp's next __syncwarp() (a shuffle orders no
+// memory), which stands before everything that relies on the word.
 __device__ __forceinline__ int ld_cta(const int *p) {
   int v;
   asm volatile("ld.acquire.cta.shared.s32 %0, [%1];\n" : "=r"(v) : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
@@ -169,6 +173,8 @@ __device__ __forceinline__ int ld_gpu(const int *p) {
 __device__ __forceinline__ void st_gpu(int *p, int v) {
   asm volatile("st.release.gpu.global.s32 [%0], %1;\n" ::"l"(p), "r"(v) : "memory");
 }
+
+__device__ __forceinline__ int of_lane0(int v) { return __shfl_sync(0xffffffffu, v, 0); }
 
 struct Shared {
   double win[kWin * kCells];     // cell c of row r at (r mod kWin) * kCells + c
@@ -375,14 +381,15 @@ __device__ __forceinline__ void rotate_chases(const ChaseArgs &Ar, Shared &S, co
   for (;;) {
     __syncwarp();
     if (!any) {
-      const int pw = ld_cta(before);
-      const int have = ld_cta(&S.loaded);
+      const int pw = of_lane0(ld_cta(before));
+      const int have = of_lane0(ld_cta(&S.loaded));
+      __syncwarp();
       int ahead = __shfl_up_sync(0xffffffffu, eff, kLanes);
       if (lane < kLanes) ahead = pw;
       if (done) eff = relay(ahead);
       run = !done && pos + lag <= ahead && pos + 4 <= have;
       if (!__any_sync(0xffffffffu, run)) {
-        if (__any_sync(0xffffffffu, have == kAborted)) break;
+        if (have == kAborted) break;
         const int last = __shfl_sync(0xffffffffu, eff, 31);
         if (last != told) {
           told = last;
@@ -415,8 +422,9 @@ __device__ __forceinline__ void rotate_chases(const ChaseArgs &Ar, Shared &S, co
         ev = __ldcg(ex + 1);
       }
     }
-    const int pw = ld_cta(before);
-    const int have = ld_cta(&S.loaded);
+    // (relied on from the next step on, behind the __syncwarp() it starts with)
+    const int pw = of_lane0(ld_cta(before));
+    const int have = of_lane0(ld_cta(&S.loaded));
     // the rotation, and beside it the step after this one for the case that
     // every bulge goes on (in one basic block, for the compiler to interleave)
     double c, s, r;
@@ -542,9 +550,9 @@ __device__ __forceinline__ void load_rows(const ChaseArgs &Ar, Shared &S, const 
   int have = base - 1, before = prev ? 0 : kFar;
   for (;;) {
     __syncwarp();
-    if (__shfl_sync(0xffffffffu, ld_cta(&S.done), 0) == kRotWarps) break;
+    if (of_lane0(ld_cta(&S.done)) == kRotWarps) break;
     if (before < kFar) {
-      before = __shfl_sync(0xffffffffu, ld_gpu(prev), 0);
+      before = of_lane0(ld_gpu(prev));
       if (before == kAborted) {
         if (lane == 0) st_cta(&S.loaded, kAborted);
         break;
@@ -554,8 +562,9 @@ __device__ __forceinline__ void load_rows(const ChaseArgs &Ar, Shared &S, const 
       if (lane == 0) st_cta(&S.before, before);
     }
     int lim = before >= N ? end : before;
-    lim = min(lim, __shfl_sync(0xffffffffu, ld_cta(&S.flushed), 0) + kWin);
+    lim = min(lim, of_lane0(ld_cta(&S.flushed)) + kWin);
     if (lim <= have) continue;
+    __syncwarp();
     for (int r0 = have + 1; r0 <= lim; r0 += 32) {
       const int r = r0 + lane;
       if (r <= lim) {
@@ -612,21 +621,20 @@ __device__ __forceinline__ void publish_rows(const ChaseArgs &Ar, Shared &S, con
   for (;;) {
     __syncwarp();
     // (the order of these loads: what is stored below was final before them)
-    const bool all = ld_cta(&S.done) == kRotWarps && ld_cta(&S.loader_done);
+    const bool all = of_lane0(ld_cta(&S.done) == kRotWarps && ld_cta(&S.loader_done));
     int least = kFar;
 #pragma unroll
     for (int w = 0; w < kRotWarps; w++) least = min(least, ld_cta(&S.least[w]));
-    const int have = ld_cta(&S.loaded);
-    const int before = ld_cta(&S.before);
-    const bool bad = have == kAborted;
-    if (__any_sync(0xffffffffu, bad)) {
-      __syncwarp();
+    least = of_lane0(least);
+    const int have = of_lane0(ld_cta(&S.loaded));
+    const int bf = of_lane0(ld_cta(&S.before));
+    __syncwarp();
+    if (have == kAborted) {
       if (lane == 0) st_gpu(word, kAborted);
       return;
     }
-    if (!__all_sync(0xffffffffu, all)) {
-      const int lim = __shfl_sync(0xffffffffu, min(min(least - 3, have), flushed + kWin), 0);
-      const int bf = __shfl_sync(0xffffffffu, before, 0);
+    if (!all) {
+      const int lim = min(min(least - 3, have), flushed + kWin);
       if (lim > flushed) {
         store_rows(Ar, S, F, flushed + 1, lim);
         flushed = lim;
@@ -645,11 +653,13 @@ __device__ __forceinline__ void publish_rows(const ChaseArgs &Ar, Shared &S, con
   }
   // the group's chases are finished: the rest of its rows, then everything
   // below is as the groups before leave it
-  store_rows(Ar, S, F, flushed + 1, ld_cta(&S.loaded));
+  const int loaded = of_lane0(ld_cta(&S.loaded));
+  __syncwarp();
+  store_rows(Ar, S, F, flushed + 1, loaded);
   __syncwarp();
   int before = prev ? 0 : kFar;
   for (long long polls = 0; before < kFar; polls++) {
-    before = __shfl_sync(0xffffffffu, ld_gpu(prev), 0);
+    before = of_lane0(ld_gpu(prev));
     if (before == kAborted || polls > max_polls) {
       if (lane == 0) {
         if (before != kAborted) atomicOr(Ar.status, ERR_STEPS);
