@@ -489,7 +489,12 @@ void bdu_thin_destroy(bdu_thin_handle h);
  *     (overlapped mixed form and mixed rank-r updates);
  *   BDU_INJECT_BHU_STALL: the first block of the BHU kernel (bdu_bhu_factor,
  *     bdu_update_bhu) leaves before its first grid barrier, and the other
- *     blocks give up a barrier wait after `value` polls.
+ *     blocks give up a barrier wait after `value` polls;
+ *   BDU_INJECT_CHASE_STALL: the first group of a chase's rotations never says
+ *     how far it is, and the rotating warps that wait for it give up after
+ *     `value` polls (not in bdu_update_batch);
+ *   BDU_INJECT_CHASE_UNDONE: it never says that it is done, and the later
+ *     groups, themselves done, give up after `value` polls (likewise).
  * In each case nothing is in flight when the waits give up; the expiry sets a
  * bit of the handle's device status word, the next synchronizing call reports
  * BDU_ETIMEOUT and the handle is poisoned.  Returns BDU_EINVAL for an unknown
@@ -499,7 +504,9 @@ enum {
   BDU_INJECT_STEP_BUDGET = 1,
   BDU_INJECT_APPLY_STALL = 2,
   BDU_INJECT_ROTVEC_STALL = 3,
-  BDU_INJECT_BHU_STALL = 4
+  BDU_INJECT_BHU_STALL = 4,
+  BDU_INJECT_CHASE_STALL = 5,
+  BDU_INJECT_CHASE_UNDONE = 6
 };
 bdu_status bdu_set_fault_injection(int site, int64_t value);
 

@@ -143,6 +143,7 @@ def load(build_if_missing: bool = True):
 
 
 INJECT_NONE, INJECT_STEP_BUDGET, INJECT_APPLY_STALL, INJECT_ROTVEC_STALL, INJECT_BHU_STALL = 0, 1, 2, 3, 4
+INJECT_CHASE_STALL, INJECT_CHASE_UNDONE = 5, 6
 
 
 def set_fault_injection(site: int, value: int = 1) -> None:

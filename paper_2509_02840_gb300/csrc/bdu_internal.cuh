@@ -99,6 +99,8 @@ struct ChaseArgs {
   int nsync;          // (of a batch's item) that number, for the staging kernel to clear
   int blocks;         // thread blocks (set by launch_chase; of a batch's item, by the caller)
   long long step_budget;  // bound on the steps of one warp for a group; 0: 64 (n + 16) + 4096
+  int stall;              // failure injection: the first group's progress word is withheld (k_chase.cu)
+  long long stall_polls;  // and its waits give up after so many polls
 };
 
 // One matrix (Q or P of one factorization) for the batched apply.

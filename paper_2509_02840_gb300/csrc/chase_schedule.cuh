@@ -83,5 +83,18 @@ BDU_HD inline bool first_op(const Phases &F, int n, int phase, int q, int &st, i
   return st != S_C || pos + 1 <= n;
 }
 
+// Watchdog: steps a warp may take for a group where the caller names none.  A
+// group needs up to about 1.3 n + 100.
+BDU_HD inline long long default_steps(int n) { return 64LL * (n + 16) + 4096; }
+// Polls of a wait before the kernel gives up.  A poll reads shared memory and
+// takes 60 cycles at least (one of the storing warp, which reads global memory,
+// 500: it has an eighth of them).  What it may have to wait for is the column:
+// about 11 n steps of 3300 cycles, behind a spike of m - n rotations of 2500;
+// and of a rank-r update every step also rotates rx later columns of U or V,
+// four at a time, every spike rotation 32 at a time, about 1500 cycles each.
+BDU_HD inline long long poll_limit(int m, int n, int rx) {
+  return default_steps(n) * (256 + 16LL * ceil_div(rx, kLanes)) + 128LL * (m - n) * (1 + ceil_div(rx, 32));
+}
+
 }  // namespace chase
 }  // namespace bdu

@@ -612,10 +612,11 @@ __device__ __forceinline__ void store_rows(const ChaseArgs &Ar, Shared &S, const
 }
 
 // Rows the group's last chase has left, back to global memory; then the
-// group's word.  fold: the last group of phase 1.
+// group's word.  fold: the last group of phase 1.  stall (failure injection):
+// 1: the word is never written, 2: it never says that the group is done.
 template <bool FAST>
 __device__ __forceinline__ void publish_rows(const ChaseArgs &Ar, Shared &S, const Phases &F, int base, const int *prev,
-                                             int *word, bool fold, long long max_polls) {
+                                             int *word, bool fold, long long max_polls, int stall) {
   const int lane = threadIdx.x & 31, n = Ar.n;
   int flushed = base - 1, told = 0;
   for (;;) {
@@ -645,7 +646,7 @@ __device__ __forceinline__ void publish_rows(const ChaseArgs &Ar, Shared &S, con
       if (f > told) {
         told = f;
         __syncwarp();
-        if (lane == 0) st_gpu(word, f);
+        if (lane == 0 && stall != 1) st_gpu(word, f);
       }
       continue;
     }
@@ -681,7 +682,7 @@ __device__ __forceinline__ void publish_rows(const ChaseArgs &Ar, Shared &S, con
       __stcg(Ar.band.r1 + j, Arith<FAST>::px(1.0, u1, __ldcg(Ar.band.r1 + j), __ldcg(Ar.band.v + j)));
   }
   __syncwarp();
-  if (lane == 0) st_gpu(word, kFar);
+  if (lane == 0 && stall != 1) st_gpu(word, stall ? F.N : kFar);
 }
 
 // The spike (m > n): one sequential chain on u in global memory, by one warp:
@@ -768,11 +769,10 @@ __device__ __forceinline__ void engine(const ChaseArgs &Ar) {
     S.tab[e] = t;
   }
   if (me < kStates) S.info[me] = geo_info(me);
-  const long long budget = 64LL * (n + 16) + 4096;
-  const int max_steps = (int)min(Ar.step_budget > 0 ? Ar.step_budget : budget, 0x7ffffffeLL);
-  // a poll takes tens of nanoseconds at least, a step half a microsecond; the
-  // spike runs before everything else
-  const long long max_polls = 256 * budget + 64LL * (m - n);
+  const int max_steps = (int)min(Ar.step_budget > 0 ? Ar.step_budget : default_steps(n), 0x7ffffffeLL);
+  const long long polls = poll_limit(m, n, Ar.rx);
+  const long long rot_polls = Ar.stall == 1 ? Ar.stall_polls : polls;
+  const long long word_polls = Ar.stall == 2 ? Ar.stall_polls : polls / 8;
   int steps = 0;  // of this warp, on the group at hand
   if (me == 0) S.far = kFar;
   for (;;) {
@@ -809,9 +809,9 @@ __device__ __forceinline__ void engine(const ChaseArgs &Ar) {
     }
     if (s == 0 && wid == 0) run_spike<FAST>(Ar);
     __syncthreads();
-    if (wid < kRotWarps) rotate_chases<FAST, EXTRA>(Ar, S, F, phase, q0, max(cnt, 0), wid, max_steps, steps, max_polls);
+    if (wid < kRotWarps) rotate_chases<FAST, EXTRA>(Ar, S, F, phase, q0, max(cnt, 0), wid, max_steps, steps, rot_polls);
     else if (wid == kRotWarps) load_rows(Ar, S, F, base, prev, s == F.g1);
-    else publish_rows<FAST>(Ar, S, F, base, prev, word, s == F.g1 - 1, max_polls / 8);
+    else publish_rows<FAST>(Ar, S, F, base, prev, word, s == F.g1 - 1, word_polls, s == 0 ? Ar.stall : 0);
     __syncthreads();
     if (S.loaded == kAborted) return;
   }
@@ -865,12 +865,16 @@ cudaError_t launch_chase_batch(const ChaseArgs *d_items, int count, int max_bloc
   return cudaGetLastError();
 }
 
-// Failure injection (BDU_INJECT_STEP_BUDGET) sets the step budget of a
-// column whose caller set none.
+// Failure injection: BDU_INJECT_STEP_BUDGET sets the step budget of a column
+// whose caller set none, BDU_INJECT_CHASE_STALL and BDU_INJECT_CHASE_UNDONE
+// withhold the first group's progress word (altogether; that it is done) and
+// set the polls after which the waits for it give up.
 cudaError_t launch_chase(const ChaseArgs &a0, cudaStream_t s) {
   ChaseArgs a = a0;
   const Injection inj = injection();
   if (a.step_budget == 0 && inj.site == BDU_INJECT_STEP_BUDGET) a.step_budget = inj.value;
+  a.stall = inj.site == BDU_INJECT_CHASE_STALL ? 1 : inj.site == BDU_INJECT_CHASE_UNDONE ? 2 : 0;
+  a.stall_polls = inj.value;
   a.blocks = a.engine == 1 ? 1 : chase_blocks(a.m, a.n);
   const cudaError_t e = cudaMemsetAsync(a.sync, 0, sizeof(int) * chase_sync_ints(a.m, a.n), s);
   if (e != cudaSuccess) return e;
