@@ -153,10 +153,10 @@ __host__ __device__ constexpr int geo_info(int st) {
 __device__ __forceinline__ int rel(int drow, int cell) { return (drow + 2) * kRowBytes + cell * 8; }
 
 // Progress words in shared memory (one CTA) and in global memory (the groups).
-// Lane 0's reading of a word counts for its warp: the lanes of a chase decide
-// alike, and what the word's writer stored before it is seen by lane 0 at once
-// and by the others after the warp's next __syncwarp() (a shuffle orders no
-// memory), which stands before everything that relies on the word.
+// What the word's writer stored before it is seen by the lane that read the
+// word at once, and by the others after the warp's next __syncwarp() (a shuffle
+// orders no memory).  The rotating warps' lanes each read the words and vote
+// (agree); in the loading and storing warps lane 0's reading counts.
 __device__ __forceinline__ int ld_cta(const int *p) {
   int v;
   asm volatile("ld.acquire.cta.shared.s32 %0, [%1];\n" : "=r"(v) : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
@@ -378,18 +378,27 @@ __device__ __forceinline__ void rotate_chases(const ChaseArgs &Ar, Shared &S, co
   int told = -1;  // last published front
   Op op = plan_any(S, st, done ? 4 : pos, q);
   bool run = false, any = false;  // may this chase's (some chase's) next op run?
+  // A chase runs when all four of its lanes say so, each by the progress words
+  // as it has read them itself.  (Lane 0's reading for the whole warp, by
+  // shuffles: a batch of 16 FP64 sessions of 64..1024 172.4 against 169.8 ms,
+  // 256 x 128 3.55 against 3.45.)
+  auto agree = [&](bool may, bool &mine) {
+    const unsigned b = __ballot_sync(0xffffffffu, may), four = b & (b >> 1) & (b >> 2) & (b >> 3) & 0x11111111u;
+    mine = (four >> (lane & ~3)) & 1;
+    return four != 0;
+  };
   for (;;) {
     __syncwarp();
     if (!any) {
-      const int pw = of_lane0(ld_cta(before));
-      const int have = of_lane0(ld_cta(&S.loaded));
-      __syncwarp();
+      const int pw = ld_cta(before);
+      const int have = ld_cta(&S.loaded);
       int ahead = __shfl_up_sync(0xffffffffu, eff, kLanes);
       if (lane < kLanes) ahead = pw;
       if (done) eff = relay(ahead);
-      run = !done && pos + lag <= ahead && pos + 4 <= have;
-      if (!__any_sync(0xffffffffu, run)) {
-        if (have == kAborted) break;
+      any = agree(!done && pos + lag <= ahead && pos + 4 <= have, run);
+      __syncwarp();
+      if (!any) {
+        if (__any_sync(0xffffffffu, have == kAborted)) break;
         const int last = __shfl_sync(0xffffffffu, eff, 31);
         if (last != told) {
           told = last;
@@ -423,8 +432,8 @@ __device__ __forceinline__ void rotate_chases(const ChaseArgs &Ar, Shared &S, co
       }
     }
     // (relied on from the next step on, behind the __syncwarp() it starts with)
-    const int pw = of_lane0(ld_cta(before));
-    const int have = of_lane0(ld_cta(&S.loaded));
+    const int pw = ld_cta(before);
+    const int have = ld_cta(&S.loaded);
     // the rotation, and beside it the step after this one for the case that
     // every bulge goes on (in one basic block, for the compiler to interleave)
     double c, s, r;
@@ -437,8 +446,8 @@ __device__ __forceinline__ void rotate_chases(const ChaseArgs &Ar, Shared &S, co
     int ahead = __shfl_up_sync(0xffffffffu, neff, kLanes);
     ahead = lane < kLanes ? pw : ahead;
     neff = done ? relay(ahead) : neff;
-    const bool nrun = !done && npos + lag <= ahead && npos + 4 <= have;
-    const bool nany = __any_sync(0xffffffffu, nrun);
+    bool nrun;
+    const bool nany = agree(!done && npos + lag <= ahead && npos + 4 <= have, nrun);
     int front = __shfl_sync(0xffffffffu, neff, 31);
     int least = __reduce_min_sync(0xffffffffu, npos);
     const bool ok = run && nz(g);
