@@ -45,4 +45,4 @@ def test_relative_accuracy(n, span, order, scale):
         assert _below(b2, Decimal(float(s)) * (1 - tol)) <= n - 1 - j, j
         assert _below(b2, Decimal(float(s)) * (1 + tol)) >= n - j, j
         checked += s < 2.0 ** -60 * sv[0]
-    assert checked or span < 20
+    assert checked or n < 9  # (the smallest orders hold no value that small)
