@@ -9,7 +9,7 @@ namespace bdu {
 
 // Device-side error bits written to the status word.
 enum : int {
-  ERR_BAND = 1,      // a write outside the stored band, or a nonzero where the schedule leaves 0
+  ERR_BAND = 1,      // the chase left a nonzero outside the matrix (non-finite entries do)
   ERR_CAP = 2,       // a chase produced more rotations than its record slot holds
   ERR_STEPS = 4,     // the chase engine exceeded its step budget (no progress)
   ERR_SCHEDULE = 8,  // an op found a zero where the schedule guarantees a nonzero

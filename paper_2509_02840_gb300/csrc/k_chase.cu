@@ -604,10 +604,20 @@ __device__ __forceinline__ void load_rows(const ChaseArgs &Ar, Shared &S, const 
   if (lane == 0) st_cta(&S.loader_done, 1);
 }
 
-__device__ __forceinline__ void store_rows(const ChaseArgs &Ar, Shared &S, const Phases &F, int r0, int r1) {
+// Rows r0..r1 back to global memory.  Returns whether one of this lane's rows
+// holds a nonzero (or a NaN) outside the matrix, which no rotation leaves there
+// while every entry is finite.
+__device__ __forceinline__ bool store_rows(const ChaseArgs &Ar, Shared &S, const Phases &F, int r0, int r1) {
   const int lane = threadIdx.x & 31, n = Ar.n, N = F.N;
+  bool outside = false;
   for (int r = r0 + lane; r <= r1; r += 32) {
     const double *d = S.win + (r & (kWin - 1)) * kCells;
+#pragma unroll
+    for (int o = 0; o < 6; o++) {
+      const int j = r + o - 2;
+      outside |= nz(d[o]) && (r > N || j < 1 || j > n);
+    }
+    outside |= (r > n && (nz(d[kR1]) || nz(d[kV]))) || (r > N && nz(d[kU]));
     if (r <= N) {
 #pragma unroll
       for (int o = 0; o < 6; o++) __stcg(Ar.band.dg[o] + r, d[o]);
@@ -618,6 +628,7 @@ __device__ __forceinline__ void store_rows(const ChaseArgs &Ar, Shared &S, const
       __stcg(Ar.band.v + r, d[kV]);
     }
   }
+  return outside;
 }
 
 // Rows the group's last chase has left, back to global memory; then the
@@ -628,6 +639,7 @@ __device__ __forceinline__ void publish_rows(const ChaseArgs &Ar, Shared &S, con
                                              int *word, bool fold, long long max_polls, int stall) {
   const int lane = threadIdx.x & 31, n = Ar.n;
   int flushed = base - 1, told = 0;
+  bool outside = false;
   for (;;) {
     __syncwarp();
     // (the order of these loads: what is stored below was final before them)
@@ -646,7 +658,7 @@ __device__ __forceinline__ void publish_rows(const ChaseArgs &Ar, Shared &S, con
     if (!all) {
       const int lim = min(min(least - 3, have), flushed + kWin);
       if (lim > flushed) {
-        store_rows(Ar, S, F, flushed + 1, lim);
+        outside |= store_rows(Ar, S, F, flushed + 1, lim);
         flushed = lim;
         __syncwarp();
         if (lane == 0) st_cta(&S.flushed, flushed);
@@ -665,7 +677,8 @@ __device__ __forceinline__ void publish_rows(const ChaseArgs &Ar, Shared &S, con
   // below is as the groups before leave it
   const int loaded = of_lane0(ld_cta(&S.loaded));
   __syncwarp();
-  store_rows(Ar, S, F, flushed + 1, loaded);
+  outside |= store_rows(Ar, S, F, flushed + 1, loaded);
+  if (outside) atomicOr(Ar.status, ERR_BAND);
   __syncwarp();
   int before = prev ? 0 : kFar;
   for (long long polls = 0; before < kFar; polls++) {
