@@ -155,8 +155,8 @@ __device__ __forceinline__ int rel(int drow, int cell) { return (drow + 2) * kRo
 // Progress words in shared memory (one CTA) and in global memory (the groups).
 // What the word's writer stored before it is seen by the lane that read the
 // word at once, and by the others after the warp's next __syncwarp() (a shuffle
-// orders no memory).  The rotating warps' lanes each read the words and vote
-// (agree); in the loading and storing warps lane 0's reading counts.
+// orders no memory).  In the loading and storing warps lane 0's reading counts,
+// among the rotating ones that of a chase's first lane.
 __device__ __forceinline__ int ld_cta(const int *p) {
   int v;
   asm volatile("ld.acquire.cta.shared.s32 %0, [%1];\n" : "=r"(v) : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
@@ -377,16 +377,7 @@ __device__ __forceinline__ void rotate_chases(const ChaseArgs &Ar, Shared &S, co
   long long polls = 0;
   int told = -1;  // last published front
   Op op = plan_any(S, st, done ? 4 : pos, q);
-  bool run = false, any = false;  // may this chase's (some chase's) next op run?
-  // A chase runs when all four of its lanes say so, each by the progress words
-  // as it has read them itself.  (Lane 0's reading for the whole warp, by
-  // shuffles: a batch of 16 FP64 sessions of 64..1024 172.4 against 169.8 ms,
-  // 256 x 128 3.55 against 3.45.)
-  auto agree = [&](bool may, bool &mine) {
-    const unsigned b = __ballot_sync(0xffffffffu, may), four = b & (b >> 1) & (b >> 2) & (b >> 3) & 0x11111111u;
-    mine = (four >> (lane & ~3)) & 1;
-    return four != 0;
-  };
+  bool may = false, any = false;  // may this chase's (some chase's) next op run?
   for (;;) {
     __syncwarp();
     if (!any) {
@@ -395,7 +386,8 @@ __device__ __forceinline__ void rotate_chases(const ChaseArgs &Ar, Shared &S, co
       int ahead = __shfl_up_sync(0xffffffffu, eff, kLanes);
       if (lane < kLanes) ahead = pw;
       if (done) eff = relay(ahead);
-      any = agree(!done && pos + lag <= ahead && pos + 4 <= have, run);
+      may = !done && pos + lag <= ahead && pos + 4 <= have;
+      any = __any_sync(0xffffffffu, may);
       __syncwarp();
       if (!any) {
         if (__any_sync(0xffffffffu, have == kAborted)) break;
@@ -419,6 +411,12 @@ __device__ __forceinline__ void rotate_chases(const ChaseArgs &Ar, Shared &S, co
     const bool rows = info & 1, has = info >= 0;
     const double f = cell_at(S, op.f), g = cell_at(S, op.g);
     const double x = cell_at(S, op.x), y = cell_at(S, op.y);
+    // A chase runs when its first lane says so, by the progress words as that
+    // lane has read them (the others follow behind the __syncwarp() above).
+    // Asked for here, beside the loads: a column of 2048, exact, 35.6 ms, of
+    // 4096, fast, 55.2 (as soon as the next step is planned: 37.1, 54.9; a
+    // vote of the four lanes there: 37.5, 55.6).
+    const bool run = __shfl_sync(0xffffffffu, (int)may, lane & ~3);
     // later columns of U (V), lane q those of number q, q + kLanes, ...: the
     // first one's entries are loaded before the rotation
     double *ex = nullptr;
@@ -446,8 +444,8 @@ __device__ __forceinline__ void rotate_chases(const ChaseArgs &Ar, Shared &S, co
     int ahead = __shfl_up_sync(0xffffffffu, neff, kLanes);
     ahead = lane < kLanes ? pw : ahead;
     neff = done ? relay(ahead) : neff;
-    bool nrun;
-    const bool nany = agree(!done && npos + lag <= ahead && npos + 4 <= have, nrun);
+    const bool nmay = !done && npos + lag <= ahead && npos + 4 <= have;
+    const bool nany = __any_sync(0xffffffffu, nmay);
     int front = __shfl_sync(0xffffffffu, neff, 31);
     int least = __reduce_min_sync(0xffffffffu, npos);
     const bool ok = run && nz(g);
@@ -494,7 +492,7 @@ __device__ __forceinline__ void rotate_chases(const ChaseArgs &Ar, Shared &S, co
       st = nst;
       op = nop;
       eff = neff;
-      run = nrun;
+      may = nmay;
       any = nany;
     } else {
       __syncwarp();
