@@ -201,7 +201,8 @@ bdu_status bdu_update_batch(bdu_handle *hs, int count, const double *const *dB, 
  * diagonal (k = 1..n-1, and k = n when m > n); right reflector k+1 zeroes row
  * k right of the superdiagonal (k = 1..n-2), so P's first column is kept.  The
  * products of the reflectors are Q_k = I - Y SL Y^T and P_k = I - W SR W^T
- * (Eq. QP with SL = 2 T^{-1}, SR = 2 R^{-1} of Eq. TR). */
+ * (Eq. QP with SL = 2 T^{-1}, SR = 2 R^{-1} of Eq. TR; after a partial run the
+ * last column of SR as bdu_bhu_factor says). */
 
 /* Sizes after `steps` iterations of Algorithm 1 (0 <= steps <= n): *kl left
  * and *kr right reflectors, kl = min(steps, n if m > n else n-1),
@@ -227,6 +228,9 @@ bdu_status bdu_bhu_sizes(int64_t m, int64_t n, int64_t steps, int64_t *kl, int64
  *        (Eq. YW; zeros above row k); W (n x kr, leading dimension n):
  *        w_2..w_{kr+1} (zeros in rows 1..k); SL (kl x kl, leading dimension
  *        kl) and SR (kr x kr, leading dimension kr), upper triangular;
+ *        after steps <= n - 2 the last column of SR holds its diagonal entry
+ *        alone, SR(1:k-1, k) = 0 for k = kr, and -2 SR(1:k-1, 1:k-1)
+ *        W(:, 1:k-1)^T W(:, k) there completes it;
  *   workspace: bdu_bhu_sizes' bytes of device memory, 16-byte aligned, owned
  *        by the caller (not kept past the call's work);
  *   stream: cudaStream_t (NULL = the legacy default stream).

@@ -614,8 +614,7 @@ __global__ void __launch_bounds__(kT, 1) k_tri_persist(BhuArgs A) {
       A.beta[j] = __ldcg(acol + j + 1);
     }
     if (!grid_barrier(A, gen)) return;
-    if (j + 1 >= A.steps) continue;
-    // the next step's p1 = R'_j W_j^T e_{j+1}
+    // R'(:, j) (after a partial run's last step too), and the next step's p1 = R'_j W_j^T e_{j+1}
     if (make && j > 0) {
       colprod(A.W, n, 0, n, j, kW, wj, A.sv);
       if (!grid_barrier(A, gen)) return;
@@ -627,7 +626,7 @@ __global__ void __launch_bounds__(kT, 1) k_tri_persist(BhuArgs A) {
       }, nullptr);
       if (gtid == 0) A.p1[j] = 2.0 * om;
       if (!grid_barrier(A, gen)) return;
-    } else if (!make && A.nr > 0) {
+    } else if (!make && A.nr > 0 && j + 1 < A.steps) {
       const int c2 = A.nr;
       rowprod<1>(A, A.SR, A.ldr, 0, c2, c2, kUT, A.W + j + 1, n, nullptr, 0, [&](int r, double s, double, double *) {
         A.p1[r] = s;
