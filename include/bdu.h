@@ -77,7 +77,7 @@ typedef struct {
                          makes that first call wait for the device; choices are kept
                          per (GPU, form, order, SMs) for the process and, if the
                          environment variable BDU_TUNE_FILE names a file, in it (JSON).
-                         FP64 form: an even number <= 64 = rows of Q/P per thread
+                         FP64 form: 2 or 4..64 = rows of Q/P per thread
                          block of the shared-memory apply.  Mixed form: 1..4 = a
                          register-resident layout of (columns x rows) per thread
                          12x8, 24x4, 6x16, 18x4; 5 = the shared-memory apply;

@@ -593,7 +593,7 @@ bdu_status tune_side(bdu_ctx *h, int side, int sm_reserve) {
   // layouts and the FP32 slab), so that the choice changes no result
   std::vector<int> cand;
   if (!mixed) {
-    for (int R : {2, 3, 4, 5, 6, 7, 8, 9, 11, 13, 16, 20, 24, 32, 48, 64}) cand.push_back(R);
+    for (int R : {2, 4, 5, 6, 7, 8, 9, 11, 13, 16, 20, 24, 32, 48, 64}) cand.push_back(R);
   } else {
     for (int v = 1; v <= 4; v++) cand.push_back(v);
     cand.push_back(kSlabVariant);
@@ -1185,7 +1185,7 @@ bdu_status bdu_create(bdu_handle *out, int64_t m, int64_t n, const double *Q, co
     return fail(nullptr, BDU_EINVAL, "bdu_create: unknown engine %d", o.engine);
   if (o.step_budget < 0) return fail(nullptr, BDU_EINVAL, "bdu_create: negative step budget");
   if (o.reorth_every < -1) return fail(nullptr, BDU_EINVAL, "bdu_create: reorth_every below -1");
-  if (o.precision == BDU_FP64 ? (o.nb < 0 || o.nb > 64 || (o.nb & 1))
+  if (o.precision == BDU_FP64 ? (o.nb < 0 || o.nb > 64 || o.nb == 1 || o.nb == 3)
                                : (o.nb < 0 || (o.nb > kSlabVariant && !is_tc_variant(o.nb))))
     return fail(nullptr, BDU_EINVAL, "bdu_create: unknown apply variant nb=%d", o.nb);
   if (!all_finite(Q, m * m) || !all_finite(P, n * n) || !all_finite(d, n) || (n > 1 && !all_finite(e, n - 1)))

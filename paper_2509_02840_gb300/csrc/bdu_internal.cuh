@@ -135,7 +135,7 @@ cudaError_t launch_project(int precision, const void *X, int64_t ld, int nrow, i
 // sm_reserve: SMs the register-resident path leaves free (for a chase that
 // runs concurrently); desc_ready: the chase descriptors of st are current.
 // variant (all give identical results): 0 = the library's choice; FP64 form:
-// R > 0 = rows per thread block of the slab kernel (even, <= 64); mixed form:
+// R > 0 = rows per thread block of the slab kernel (2..64); mixed form:
 // 1..4 = a register layout of launch_apply_reg, kSlabVariant = the slab
 // kernel.  cudaErrorNotSupported when the variant does not cover the shape.
 // gate (slab kernel only; may be null): a device error word; when an earlier
