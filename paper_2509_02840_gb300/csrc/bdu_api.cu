@@ -514,13 +514,17 @@ namespace tune {
 std::mutex mu;
 std::map<std::string, int> table;
 bool loaded = false;
+// In the FP64 form's keys: which version of its apply kernel a height was timed
+// with (none: rotations of both rows and columns a thread, even heights only).
+// A file may hold heights that were the best of an earlier one.
+constexpr const char *kSlab64 = "|items16";
 
 std::string key(const bdu_ctx *h, int dim, int sm_reserve) {
   cudaDeviceProp p{};
   cudaGetDeviceProperties(&p, h->device);
   char buf[512];
-  snprintf(buf, sizeof buf, "%s|%s|%d|%d", p.name, h->opt.precision == BDU_FP64 ? "fp64" : "mixed", dim,
-           sm_reserve);
+  const bool fp64 = h->opt.precision == BDU_FP64;
+  snprintf(buf, sizeof buf, "%s|%s|%d|%d%s", p.name, fp64 ? "fp64" : "mixed", dim, sm_reserve, fp64 ? kSlab64 : "");
   for (char *c = buf; *c; c++)
     if (*c == '"' || *c == '\\') *c = '_';
   return buf;
