@@ -31,25 +31,14 @@ namespace {
 constexpr int kThreads = 512;
 constexpr int kPer = 5;  // rotations per thread per chase held in registers
 
-template <typename T> struct Coef;
-template <> struct Coef<double> {
-  double c, s;
-  static __device__ __forceinline__ Coef load(const RotStream &st, int side, size_t i) {
-    Coef k;
-    k.c = side == 0 ? st.Lc[i] : st.Rc[i];
-    k.s = side == 0 ? st.Ls[i] : st.Rs[i];
-    return k;
-  }
-  static __device__ __forceinline__ Coef load_spike(const RotStream &st, int i) {
-    Coef k; k.c = st.Sc[i]; k.s = st.Ss[i]; return k;
-  }
-  __device__ __forceinline__ void rot(double &x, double &y) const {
-    const double xo = x, yo = y;
-    x = __dadd_rn(__dmul_rn(c, xo), __dmul_rn(s, yo));
-    y = __dadd_rn(__dmul_rn(-s, xo), __dmul_rn(c, yo));
-  }
-};
-template <> struct Coef<float> {
+// One FP64 rotation of a pair.
+__device__ __forceinline__ void rot64(double c, double s, double &x, double &y) {
+  const double xo = x, yo = y;
+  x = __dadd_rn(__dmul_rn(c, xo), __dmul_rn(s, yo));
+  y = __dadd_rn(__dmul_rn(-s, xo), __dmul_rn(c, yo));
+}
+// One FP32 rotation, as recorded.
+struct Coef {
   float c, s;
   static __device__ __forceinline__ Coef load(const RotStream &st, int side, size_t i) {
     const float2 v = side == 0 ? st.Lf[i] : st.Rf[i];
@@ -66,34 +55,18 @@ template <> struct Coef<float> {
   }
 };
 
-// 16-byte vectors of the tile: 4 floats or 2 doubles
-template <typename T> struct Vec;
-template <> struct Vec<float> {
-  using type = float4;
-  static constexpr int V = 4;
-  static __device__ __forceinline__ void rot(const Coef<float> &k, float4 &x, float4 &y) {
-    k.rot(x.x, y.x); k.rot(x.y, y.y); k.rot(x.z, y.z); k.rot(x.w, y.w);
-  }
-};
-template <> struct Vec<double> {
-  using type = double2;
-  static constexpr int V = 2;
-  static __device__ __forceinline__ void rot(const Coef<double> &k, double2 &x, double2 &y) {
-    k.rot(x.x, y.x); k.rot(x.y, y.y);
-  }
-};
+constexpr int kVec = 4;  // floats of a 16-byte vector of the tile
+__device__ __forceinline__ void rot_vec(const Coef &k, float4 &x, float4 &y) {
+  k.rot(x.x, y.x); k.rot(x.y, y.y); k.rot(x.z, y.z); k.rot(x.w, y.w);
+}
 
 // Shared-memory tile: column-major, column c's R rows at tile[c*csw ...],
-// csw = V * (odd count of 16-byte vectors) >= R, so that the columns touched
+// csw = kVec * (odd count of 16-byte vectors) >= R, so that the columns touched
 // by a stride-3 chase fall in distinct 16-byte bank groups.
-template <typename T>
-__device__ __forceinline__ void apply_slab_body(T *__restrict__ X, int64_t ld, int nrow, int ncol, int R,
-                                                int csw, const RotStream &st, int side, int with_spike,
-                                                int slab, int *status) {
-  using VT = typename Vec<T>::type;
-  constexpr int V = Vec<T>::V;
+__device__ __forceinline__ void apply_slab32(float *__restrict__ X, int64_t ld, int nrow, int ncol, int R, int csw,
+                                             const RotStream &st, int side, int with_spike, int slab, int *status) {
   extern __shared__ __align__(16) unsigned char raw[];
-  T *tile = reinterpret_cast<T *>(raw);
+  float *tile = reinterpret_cast<float *>(raw);
   const int r0 = slab * R;
   const int rows = min(R, nrow - r0);
   if (rows <= 0) return;
@@ -101,28 +74,28 @@ __device__ __forceinline__ void apply_slab_body(T *__restrict__ X, int64_t ld, i
   const int32_t *Ca = side == 0 ? st.La : st.Ra;
   const int32_t *Cn = side == 0 ? st.Ln : st.Rn;
   const int cap = st.cap, ntask = st.T;
-  const int nv = R / V;  // vectors per column
+  const int nv = R / kVec;  // vectors per column
 
   for (int64_t q = tid; q < (int64_t)R * ncol; q += kThreads) {
     const int col = (int)(q / R), rr = (int)(q % R);
-    tile[(size_t)col * csw + rr] = (rr < rows) ? X[(size_t)col * ld + r0 + rr] : T(0);
+    tile[(size_t)col * csw + rr] = (rr < rows) ? X[(size_t)col * ld + r0 + rr] : 0.f;
   }
   __syncthreads();
 
   if (with_spike) {
     const int ns = st.Sn[0];
     if (tid < rows) {
-      T *row = tile + tid;
+      float *row = tile + tid;
       for (int e = 0; e < ns; e++) {
         const int a = st.Sa[e] - 1;  // 0-based first column of the pair
-        Coef<T>::load_spike(st, e).rot(row[(size_t)a * csw], row[(size_t)(a + 1) * csw]);
+        Coef::load_spike(st, e).rot(row[(size_t)a * csw], row[(size_t)(a + 1) * csw]);
       }
     }
     __syncthreads();
   }
 
   // the rotations of the current chase owned by this thread, in registers
-  Coef<T> cf[kPer];
+  Coef cf[kPer];
   int ca[kPer];
   int cnt = ntask > 0 ? Cn[0] : 0;
 #pragma unroll
@@ -130,13 +103,13 @@ __device__ __forceinline__ void apply_slab_body(T *__restrict__ X, int64_t ld, i
     const int e = tid + k * kThreads;
     ca[k] = -1;
     if (e < cnt) {
-      cf[k] = Coef<T>::load(st, side, (size_t)e);
+      cf[k] = Coef::load(st, side, (size_t)e);
       ca[k] = Ca[e] - 1;
     }
   }
   for (int t = 0; t < ntask; t++) {
     // prefetch chase t+1
-    Coef<T> nf[kPer];
+    Coef nf[kPer];
     int na[kPer];
     const int ncnt = (t + 1 < ntask) ? Cn[t + 1] : 0;
     const size_t nbase = (size_t)(t + 1) * cap;
@@ -145,7 +118,7 @@ __device__ __forceinline__ void apply_slab_body(T *__restrict__ X, int64_t ld, i
       const int e = tid + k * kThreads;
       na[k] = -1;
       if (e < ncnt) {
-        nf[k] = Coef<T>::load(st, side, nbase + e);
+        nf[k] = Coef::load(st, side, nbase + e);
         na[k] = Ca[nbase + e] - 1;
       }
     }
@@ -153,11 +126,11 @@ __device__ __forceinline__ void apply_slab_body(T *__restrict__ X, int64_t ld, i
 #pragma unroll
     for (int k = 0; k < kPer; k++) {
       if ((unsigned)ca[k] < (unsigned)(ncol - 1)) {
-        VT *pa = reinterpret_cast<VT *>(tile + (size_t)ca[k] * csw);
-        VT *pb = reinterpret_cast<VT *>(tile + (size_t)(ca[k] + 1) * csw);
+        float4 *pa = reinterpret_cast<float4 *>(tile + (size_t)ca[k] * csw);
+        float4 *pb = reinterpret_cast<float4 *>(tile + (size_t)(ca[k] + 1) * csw);
         for (int q = 0; q < nv; q++) {
-          VT x = pa[q], y = pb[q];
-          Vec<T>::rot(cf[k], x, y);
+          float4 x = pa[q], y = pb[q];
+          rot_vec(cf[k], x, y);
           pa[q] = x;
           pb[q] = y;
         }
@@ -169,17 +142,17 @@ __device__ __forceinline__ void apply_slab_body(T *__restrict__ X, int64_t ld, i
     const int ccnt = Cn[t];
     for (int e = tid + kPer * kThreads; e < ccnt; e += kThreads) {
       const size_t i = (size_t)t * cap + e;
-      const Coef<T> k = Coef<T>::load(st, side, i);
+      const Coef k = Coef::load(st, side, i);
       const int a = Ca[i] - 1;
       if ((unsigned)a >= (unsigned)(ncol - 1)) {
         if (status) atomicOr(status, ERR_RANGE);
         continue;
       }
-      VT *pa = reinterpret_cast<VT *>(tile + (size_t)a * csw);
-      VT *pb = reinterpret_cast<VT *>(tile + (size_t)(a + 1) * csw);
+      float4 *pa = reinterpret_cast<float4 *>(tile + (size_t)a * csw);
+      float4 *pb = reinterpret_cast<float4 *>(tile + (size_t)(a + 1) * csw);
       for (int q = 0; q < nv; q++) {
-        VT x = pa[q], y = pb[q];
-        Vec<T>::rot(k, x, y);
+        float4 x = pa[q], y = pb[q];
+        rot_vec(k, x, y);
         pa[q] = x;
         pb[q] = y;
       }
@@ -261,7 +234,7 @@ __device__ __forceinline__ void apply_slab64(double *__restrict__ X, int64_t ld,
         const int en = min(e + 1, ns - 1);  // the next rotation, while this one is applied
         const double nc = st.Sc[en], nsn = st.Ss[en];
         const int na = st.Sa[en] - 1;
-        Coef<double>{c, s}.rot(row[(size_t)a * csw], row[(size_t)(a + 1) * csw]);
+        rot64(c, s, row[(size_t)a * csw], row[(size_t)(a + 1) * csw]);
         c = nc; s = nsn; a = na;
       }
     }
@@ -367,7 +340,7 @@ __global__ void __launch_bounds__(kThreads) k_apply_slab(T *__restrict__ X, int6
                                                          int side, int with_spike, int *status, const int *gate) {
   if (gate && *(volatile const int *)gate) return;
   if constexpr (sizeof(T) == 8) apply_slab64(X, ld, nrow, ncol, R, csw, st, side, with_spike, blockIdx.x, status);
-  else apply_slab_body<T>(X, ld, nrow, ncol, R, csw, st, side, with_spike, blockIdx.x, status);
+  else apply_slab32(X, ld, nrow, ncol, R, csw, st, side, with_spike, blockIdx.x, status);
 }
 
 // Many matrices of uneven sizes in one launch: block b works on the slab
@@ -388,8 +361,8 @@ __global__ void __launch_bounds__(kThreads) k_apply_batch(const ApplyItem *__res
     apply_slab64((T *)it.X, it.ld, it.nrow, it.ncol, it.R, it.csw, it.st, it.side, it.with_spike, b - first[lo],
                  it.status);
   else
-    apply_slab_body<T>((T *)it.X, it.ld, it.nrow, it.ncol, it.R, it.csw, it.st, it.side, it.with_spike,
-                       b - first[lo], it.status);
+    apply_slab32((T *)it.X, it.ld, it.nrow, it.ncol, it.R, it.csw, it.st, it.side, it.with_spike, b - first[lo],
+                 it.status);
 }
 
 }  // namespace
