@@ -201,7 +201,7 @@ CHASE_FLOPS_PER_ROTATION = 26
 # ncu capture (one pass) of a dense rank-1 update with the chase kernel as it is:
 # the rotation records written (FP32 (c, s) and an int32 pair index per rotation,
 # 12 B x 25.2M = 302 MB, part of which is still in L2 when the launch ends).
-CHASE_TRAFFIC_4096 = 3.19e6 + 247.32e6
+CHASE_TRAFFIC_4096 = 3.09e6 + 247.48e6
 
 
 def roofline(st, precision, rotations_per_update, launches_per_update, steps_per_update=None):
@@ -221,7 +221,8 @@ def roofline(st, precision, rotations_per_update, launches_per_update, steps_per
         if steps_per_update:
             # the kernel is bound by its chain of dependent steps, not by a throughput
             out["critical_path"] = {"steps_per_launch": steps_per_update,
-                                    "us_per_step": per_launch_ms * 1e3 / steps_per_update}
+                                    "us_per_step": per_launch_ms * 1e3 / steps_per_update,
+                                    "steps_are": "the longest chain of dependent rotations by the schedule, not counted"}
         return out
     # apply: algorithmic bytes = one read + one write of Q and P per rank-1 column
     es = 8 if precision == 0 else 4
@@ -749,7 +750,7 @@ def run_network(args):
                        "l2": "not flushed: each update streams > 10 GB"},
             "apply_variant": st["apply_variant"], "orthogonality": {"q": q, "p": p, "tolerance": 1e-5},
             "kernel_ms_per_update": {k: st["ms_" + k] / tu for k in ("project", "chase", "apply_q", "apply_p")},
-            "chase_steps_per_update": (st["chase_steps"] - st0["chase_steps"]) / K,
+            "rotations_tried_per_update": (st["chase_steps"] - st0["chase_steps"]) / K,
             "clocks": clk, "cpu_baseline": None,
             "note": "no CPU baseline: the oracle does not finish an update at this size in minutes"}
     print(json.dumps(line), flush=True)

@@ -182,7 +182,10 @@ bdu_status bdu_update_dev(bdu_handle h, const double *dB, const double *dC, int6
  * (round k serves the items with r[i] > k); each round is one launch of each
  * kernel kind -- projection (first round), staging, bulge chasing (the thread
  * blocks of every factorization) and a fused apply whose blocks cover the row slabs
- * of every Q and P in the round.  The results are identical to bdu_update_dev
+ * of every Q and P in the round.  BDU_MIXED: the rotations of an item's later
+ * projections, the blocked applies of orders from 1024 on and the
+ * re-orthogonalizations are the item's own launches, on its handle's stream
+ * beside the other items'.  The results are identical to bdu_update_dev
  * on each handle.  All handles must share a device and precision and appear
  * once.  stream: cudaStream_t for the batch (NULL = the first handle's); the
  * batch is ordered after each handle's queued work and each handle's later

@@ -298,7 +298,8 @@ cudaError_t enqueue_probe(bdu_ctx *h, int which, double *dst, cudaStream_t s) {
 }
 
 // ---- overlapped mixed form -------------------------------------------------
-// SMs an overlapped apply leaves to the concurrent chase.
+// SMs an overlapped register apply leaves to the concurrent chase, which has up
+// to 10 blocks at the orders (below kBlockedFrom) where that apply runs.
 constexpr int kChaseSMs = 16;
 
 // Enqueues on the apply stream the application of record buffer buf to Q and

@@ -43,8 +43,8 @@
 // number of FP64 instructions in one warp's chain.  Each chase therefore has
 // kLanes = 4 lanes: the rotation is computed by all four at once (c, s and r,
 // products or quotients with one factor in common, in one instruction), and
-// each lane rotates one of the up to four pairs: 12 FP64 instructions a step
-// (16 + 10 with a lane per chase).  A fifth warp loads rows, a sixth stores
+// each lane rotates one of the up to four pairs: 12 FP64 instructions a step in
+// the fast form (16 + 10 with a lane per chase), 22 in the exact one.  A fifth warp loads rows, a sixth stores
 // them and publishes the group's word.  Groups are taken from a ticket
 // counter in order, so a block that waits for the group before it waits for
 // one that is already running: any number of resident blocks makes progress.
@@ -228,7 +228,7 @@ __device__ __forceinline__ double rsqrt_f64(double q) {
 // the rounding interval around it through its exact remainder: h is the
 // rounded root of q iff q - h^2 lies in (-h ulp, h ulp], a quotient the
 // rounded one iff its remainder is below half an ulp of it times h (a tie
-// cannot occur).  18 FP64 instructions: the rotation took 4.4k cycles at n =
+// cannot occur).  16 FP64 instructions: the rotation took 4.4k cycles at n =
 // 1024 with the library's square root and division and takes 1.8k.  The scaling by
 // the larger exponent is exact and does not change any rounding while both
 // inputs lie within 2^-500..2^500 and within 2^900 of each other; for others
@@ -854,7 +854,7 @@ int chase_sync_ints(int m, int n) {
 // hand-over between groups.  A block that holds the ticket of a later group
 // keeps its SM from the application that runs beside the chase: at 4096, 67
 // blocks 83.9 ms an overlapped update, 35 blocks 75.5, 24 blocks 76.3 (the
-// chase alone 54.2, 54.3, 56).
+// chase alone 54.2, 54.3, 56).  (Measured at 4096 in the fast form only.)
 int chase_blocks(int m, int n) {
   const Phases F = phases_of(m, n);
   return std::min(F.g1 + F.g2 + F.g3, n / (4 * kGroup) + 3);
